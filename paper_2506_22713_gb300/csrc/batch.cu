@@ -510,8 +510,9 @@ __host__ __device__ inline PLayout playout(int64_t mmax, int64_t nmax) {
 
 __device__ __noinline__ void leaf(const double *G, int w, int decide, double eps2, double delta_coef, double rho,
                                      double *R, double *Ri, int *info, double ni_tau2, unsigned char *sm) {
-    chol_leaf_cta<true>(G, kPRcap, w, decide, eps2, delta_coef, rho, 0.0, R, kPRcap, Ri, kPRcap, info, ni_tau2,
-                        (double *)sm);
+    const LeafArgs a{G, kPRcap, w, decide, eps2, delta_coef, rho, 0.0, R, kPRcap, Ri, kPRcap, nullptr, 0, info, ni_tau2,
+                     nullptr, nullptr};
+    chol_leaf_cta<true>(a, (double *)sm);
     __syncthreads();
 }
 // Per-phase cycle accounting of the measurement hook: thread 0 adds the

@@ -1,11 +1,12 @@
-// Small dense factorisations in FP64, one CTA each:
+// Small dense factorisations in FP64:
 //  * Cholesky of a w x w Gram matrix (w <= 128) with the rank test of
 //    Alg. 1 steps 6-11 folded into the pivot loop, plus the inverse of the
-//    triangular factor (CholQR: P = Y R^{-1}) -- the leaf itself, and its
-//    rank decisions, are in chol_leaf.cuh;
-//  * the diagonal of T = R2 R1 (the T_j(l,l) the test reads, Rem. 3.6);
+//    triangular factor (CholQR: P = Y R^{-1}) and the diagonal of T = R2 R1
+//    (the T_j(l,l) the test reads, Rem. 3.6) -- the leaf, on one CTA
+//    (chol_leaf.cuh) or, for wide blocks, a cluster (chol_block.cuh);
 //  * trace(G) for the shift of shifted CholQR.
 #include "common.cuh"
+#include "chol_block.cuh"
 #include "chol_leaf.cuh"
 #include "instrument.cuh"
 
@@ -14,26 +15,17 @@
 namespace eod {
 namespace {
 
+// One CTA, column by column: LA the schedule with one barrier per pivot, else
+// the one with two (decide | 256 of the test hook).
 template <bool LA>
-__global__ void __launch_bounds__(kLeafThreads) chol_small_kernel(const double *__restrict__ G, int64_t ldg, int w,
-                                                                  int decide, double eps2, double delta_coef,
-                                                                  double rho, double shift, double *__restrict__ R,
-                                                                  int64_t ldr, double *__restrict__ Rinv,
-                                                                  int64_t ldinv, int *info, double ni_tau2) {
+__global__ void __launch_bounds__(kLeafThreads) chol_small_kernel(const LeafArgs A) {
     extern __shared__ double sh[];
-    chol_leaf_cta<LA>(G, ldg, w, decide, eps2, delta_coef, rho, shift, R, ldr, Rinv, ldinv, info, ni_tau2, sh);
+    chol_leaf_cta<LA>(A, sh);
 }
 
 __global__ void recip_kernel(const double *d, double *out, int64_t n) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = recip_pos(d[i]);
-}
-
-__global__ void tdiag_kernel(const double *R1, const double *R2, int64_t ldr, const int *p_dev,
-                             double *tdiag) {
-    const int p = *p_dev;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < p; j += gridDim.x * blockDim.x)
-        tdiag[j] = fabs(R1[j + j * ldr] * R2[j + j * ldr]);
 }
 
 // ||G - I||_F^2 of a symmetric p x p matrix from its upper triangle.
@@ -92,20 +84,33 @@ __global__ void trace_kernel(const double *G, int64_t ldg, int64_t p, double *ou
 
 cudaError_t chol_small(const double *G, int64_t ldg, int w, int decide, double eps2, double delta_coef,
                        double rho, double shift, double *R, int64_t ldr, double *Rinv, int64_t ldinv, int *info,
-                       cudaStream_t s, double ni_tau2, bool classic) {
+                       cudaStream_t s, double ni_tau2, bool classic, const CholOut &out) {
     if (w < 1 || w > 128) return cudaErrorInvalidValue;
     if (decide || shift != 0.0) ni_tau2 = 0.0;
-    EOD_CUDA_TRY(set_smem_once(chol_small_kernel<true>, (int)leaf_smem_bytes(128)));
-    EOD_CUDA_TRY(set_smem_once(chol_small_kernel<false>, (int)leaf_smem_bytes(128)));
     ProfScope prof(PROF_CHOL, (double)w * w * w * (Rinv ? 2.0 : 1.0) / 3.0, sizeof(double) * 3.0 * w * w, s);
     count_launch();
-    if (classic)
-        chol_small_kernel<false><<<1, kLeafThreads, leaf_smem_bytes(w), s>>>(G, ldg, w, decide, eps2, delta_coef, rho,
-                                                                            shift, R, ldr, Rinv, ldinv, info, ni_tau2);
-    else
-        chol_small_kernel<true><<<1, kLeafThreads, leaf_smem_bytes(w), s>>>(G, ldg, w, decide, eps2, delta_coef, rho,
-                                                                           shift, R, ldr, Rinv, ldinv, info, ni_tau2);
-    return cudaGetLastError();
+    const LeafArgs args{G, ldg, w, decide, eps2, delta_coef, rho, shift, R, ldr, Rinv, ldinv, out.RinvF, out.ldf, info,
+                        ni_tau2, out.tR1, out.tdiag};
+    if (classic || w <= kLeafOneCta) {
+        auto kern = classic ? chol_small_kernel<false> : chol_small_kernel<true>;
+        EOD_CUDA_TRY(set_smem_once(kern, (int)leaf_smem_bytes(128)));
+        kern<<<1, kLeafThreads, leaf_smem_bytes(w), s>>>(args);
+        return cudaGetLastError();
+    }
+    constexpr int C = kLeafCluster;
+    EOD_CUDA_TRY(set_smem_once(chol_block_kernel, (int)block_leaf_smem_bytes(128)));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(kLeafThreads);
+    cfg.dynamicSmemBytes = block_leaf_smem_bytes(w);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, chol_block_kernel, args);
 }
 
 cudaError_t offidentity_sumsq(const double *G, int64_t ldg, int64_t p, double *part, double *out, cudaStream_t s) {
@@ -122,13 +127,6 @@ cudaError_t near_identity_factor(const double *G, int64_t ldg, int64_t p, double
     const int64_t tot = p * p;
     near_identity_kernel<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, s>>>(G, ldg, p, R, ldr, RiD,
                                                                                                 pb);
-    return cudaGetLastError();
-}
-
-cudaError_t tdiag_product(const double *R1, const double *R2, int64_t ldr, const int *p_dev, double *tdiag,
-                          cudaStream_t s) {
-    count_launch();
-    tdiag_kernel<<<1, 128, 0, s>>>(R1, R2, ldr, p_dev, tdiag);
     return cudaGetLastError();
 }
 

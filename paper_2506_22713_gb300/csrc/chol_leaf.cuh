@@ -99,6 +99,23 @@ __device__ __forceinline__ void ldl_pivot(const double *S, int ld, int w, int j,
 
 constexpr int kLeafThreads = 512;
 
+struct LeafArgs {
+    const double *G;
+    int64_t ldg;
+    int w, decide;
+    double eps2, delta_coef, rho, shift;
+    double *R;
+    int64_t ldr;
+    double *Rinv;          // may be null
+    int64_t ldinv;
+    float *RinvF;          // may be null: R^{-1} rounded to FP32 (ld ldf)
+    int64_t ldf;
+    int *info;
+    double ni_tau2;
+    const double *tR1;     // may be null: tdiag[j] = |tR1(j, j) R(j, j)|, ld ldr
+    double *tdiag;
+};
+
 inline size_t leaf_smem_bytes(int w) {
     // S, M, pivots, sqrt and 1/sqrt, three key arrays, the entry table, then
     // (8-byte aligned) the lookahead's second M buffer
@@ -135,9 +152,13 @@ inline size_t leaf_smem_bytes(int w) {
 // and info may point to shared or global memory.  Every thread of the CTA
 // must call it; it ends without a trailing barrier.
 template <bool LA>
-__device__ void chol_leaf_cta(const double *__restrict__ G, int64_t ldg, int w, int decide, double eps2,
-                              double delta_coef, double rho, double shift, double *__restrict__ R, int64_t ldr,
-                              double *__restrict__ Rinv, int64_t ldinv, int *info, double ni_tau2, double *sh) {
+__device__ void chol_leaf_cta(const LeafArgs &A, double *sh) {
+    const double *__restrict__ G = A.G;
+    double *__restrict__ R = A.R, *__restrict__ Rinv = A.Rinv;
+    const int64_t ldg = A.ldg, ldr = A.ldr, ldinv = A.ldinv;
+    const int w = A.w, decide = A.decide;
+    const double eps2 = A.eps2, delta_coef = A.delta_coef, rho = A.rho, shift = A.shift, ni_tau2 = A.ni_tau2;
+    int *info = A.info;
     constexpr int NT = kLeafThreads;
     // Near-identity Gram (the second pass of CholQR2, G = P^T P = I + E with
     // P already orthonormal to first order): when ||E||_F^2 <= ni_tau2,
@@ -159,8 +180,11 @@ __device__ void chol_leaf_cta(const double *__restrict__ G, int64_t ldg, int w, 
                 for (int i = ln; i < w; i += 32) {
                     const double g = (i <= c) ? G[i + (int64_t)c * ldg] : 0.0;
                     const double x = (i < c) ? g : (i == c ? 0.5 * (g - 1.0) : 0.0);
-                    R[i + (int64_t)c * ldr] = (i == c ? 1.0 : 0.0) + x;
-                    if (Rinv) Rinv[i + (int64_t)c * ldinv] = (i == c ? 1.0 : 0.0) - x;
+                    const double one = i == c ? 1.0 : 0.0;
+                    R[i + (int64_t)c * ldr] = one + x;
+                    if (Rinv) Rinv[i + (int64_t)c * ldinv] = one - x;
+                    if (A.RinvF) A.RinvF[i + (int64_t)c * A.ldf] = (float)(one - x);
+                    if (A.tdiag && i == c) A.tdiag[c] = fabs(A.tR1[c + (int64_t)c * ldr] * (one + x));
                 }
             if (threadIdx.x == 0) {
                 info[0] = w;
@@ -353,6 +377,7 @@ __device__ void chol_leaf_cta(const double *__restrict__ G, int64_t ldg, int w, 
         const double s = sqrt(dv[j]);
         sq[j] = s;
         rs[j] = 1.0 / s;
+        if (A.tdiag) A.tdiag[j] = fabs(A.tR1[j + (int64_t)j * ldr] * s);
     }
     __syncthreads();
     // R(i, c) = u_i(c) / sqrt(d_i) for i < c, sqrt(d_i) on the diagonal;
@@ -362,7 +387,9 @@ __device__ void chol_leaf_cta(const double *__restrict__ G, int64_t ldg, int w, 
         int c = tid / p, i = tid - c * p;
         for (int e = tid; e < tot; e += NT) {
             R[i + (int64_t)c * ldr] = (i < c) ? S[i + c * ld] * rs[i] : (i == c ? sq[i] : 0.0);
-            if (Rinv) Rinv[i + (int64_t)c * ldinv] = (i < c) ? S[c + i * ld] * rs[c] : (i == c ? rs[c] : 0.0);
+            const double z = (i < c) ? S[c + i * ld] * rs[c] : (i == c ? rs[c] : 0.0);
+            if (Rinv) Rinv[i + (int64_t)c * ldinv] = z;
+            if (A.RinvF) A.RinvF[i + (int64_t)c * A.ldf] = (float)z;
             c += dc;
             i += di;
             if (i >= p) { i -= p; ++c; }

@@ -261,8 +261,18 @@ cudaError_t gram_tiled_f32(const float *W, int64_t rows, int64_t p, int64_t ldw,
 // --------------------------------------------------------------------------
 enum CholCode { CHOL_ALL = 0, CHOL_BELOW = 1, CHOL_UNCERTAIN = 2, CHOL_FAIL = 3 };
 
-// Cholesky G = R^T R of the w x w matrix G (upper triangle read, FP64; one
-// CTA, computed as L D L^T) with the rank decision of Alg. 1 steps 6-11 when
+// Further outputs of a leaf: R^{-1} rounded to FP32, and the diagonal of
+// T = R2 R1 when the factor is the second pass's R2: tdiag[j] =
+// |tR1(j, j) R(j, j)|, R1 with R's leading dimension.
+struct CholOut {
+    float *RinvF = nullptr;
+    int64_t ldf = 0;
+    const double *tR1 = nullptr;
+    double *tdiag = nullptr;
+};
+
+// Cholesky G = R^T R of the w x w matrix G (upper triangle read, FP64,
+// computed as L D L^T) with the rank decision of Alg. 1 steps 6-11 when
 // decide != 0:
 //   info[0] = p (leading columns factored), info[1] = CholCode,
 // R (p x p upper, ld ldr) and its inverse Rinv (ld ldr); the original
@@ -274,7 +284,7 @@ enum CholCode { CHOL_ALL = 0, CHOL_BELOW = 1, CHOL_UNCERTAIN = 2, CHOL_FAIL = 3 
 cudaError_t chol_small(const double *G, int64_t ldg, int w, int decide, double eps2,
                        double delta_coef, double rho, double shift, double *R, int64_t ldr,
                        double *Rinv, int64_t ldinv, int *info, cudaStream_t s, double ni_tau2 = 0.0,
-                       bool classic = false);
+                       bool classic = false, const CholOut &out = CholOut());
 // out[0] = ||G - I||_F^2 of the symmetric p x p matrix G (upper triangle
 // read), through kOffIdMaxBlocks partial sums in `part`
 constexpr int kOffIdMaxBlocks = 608;
@@ -284,9 +294,6 @@ cudaError_t offidentity_sumsq(const double *G, int64_t ldg, int64_t p, double *p
 // of width pb at RiD + J pb^2 (ld pb)
 cudaError_t near_identity_factor(const double *G, int64_t ldg, int64_t p, double *R, int64_t ldr, double *RiD,
                                  int pb, cudaStream_t s);
-// tdiag[j] = |R1(j,j) * R2(j,j)|, j < p
-cudaError_t tdiag_product(const double *R1, const double *R2, int64_t ldr, const int *p_dev,
-                          double *tdiag, cudaStream_t s);
 // trace(G) for the shift of shifted CholQR
 cudaError_t trace_sum(const double *G, int64_t ldg, int64_t p, double *out, cudaStream_t s);
 

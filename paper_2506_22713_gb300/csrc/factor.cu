@@ -571,6 +571,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     };
 
     // ---- Alg. 1 ----
+    constexpr bool f32 = std::is_same<T, float>::value;   // the leaves then write R^{-1} in FP32 (RinvT) alone
     const double eps2 = eps * eps;
     const double delta_coef = 64.0 * ((double)k + std::sqrt((double)m)) * kU64;
     GemmExtra ex, sym, bup;
@@ -713,7 +714,10 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             }
             // step 5 (pass 1) + steps 6-11: Gram, Cholesky with the rank test
             EOD_CU(gram_skinny<T>(Yc, m, (int)wdt, m, G, k, &ws, s));
-            EOD_CU(chol_small(G, k, (int)wdt, 1, eps2, delta_coef, Traits<T>::rho, 0.0, R1, k, R1i, k, info, s));
+            CholOut o1;
+            if (f32) o1.RinvF = (float *)RinvT, o1.ldf = k;
+            EOD_CU(chol_small(G, k, (int)wdt, 1, eps2, delta_coef, Traits<T>::rho, 0.0, R1, k, f32 ? nullptr : R1i, k,
+                              info, s, 0.0, false, o1));
             EOD_CU(cudaMemcpyAsync(hm.info, info, sizeof(int) * 2, cudaMemcpyDeviceToHost, s));
             if (launch_ahead) {
                 const int64_t c1 = kept_block + f, f1 = std::min(k, cap - c1);
@@ -730,22 +734,18 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             const int p = hm.info[0], code = hm.info[1];
             if (p > 0) {
                 // P1 = Y(:,1:p) R1^{-1}; pass 2: G2 = P1^T P1 = R2^T R2; P = P1 R2^{-1}
-                const T *Ri = (const T *)R1i;
-                if (!std::is_same<T, double>::value) {
-                    EOD_CU((copy_matrix<double, T>(R1i, k, RinvT, k, p, p, false, s)));
-                    Ri = RinvT;
-                }
+                const T *Ri = f32 ? (const T *)RinvT : (const T *)R1i;
                 EOD_CU((gemm<T, T, T, T>(false, false, m, p, p, 1.0, Yc, m, Ri, k, 0.0, T1, m, bup, &ws, s)));
                 EOD_CU(gram_skinny<T>(T1, m, p, m, G, k, &ws, s));
                 int *pinf = pinfo + 2 * (int64_t)panel_p.size();
-                EOD_CU(chol_small(G, k, p, 0, 0.0, 0.0, 0.0, 0.0, R2, k, R2i, k, pinf, s, near_id_tau2<T>()));
-                const T *Ri2 = (const T *)R2i;
-                if (!std::is_same<T, double>::value) {
-                    EOD_CU((copy_matrix<double, T>(R2i, k, RinvT, k, p, p, false, s)));
-                    Ri2 = RinvT;
-                }
+                CholOut o2;
+                if (f32) o2.RinvF = (float *)RinvT, o2.ldf = k;
+                o2.tR1 = R1;
+                o2.tdiag = tdiag_d + nt;
+                EOD_CU(chol_small(G, k, p, 0, 0.0, 0.0, 0.0, 0.0, R2, k, f32 ? nullptr : R2i, k, pinf, s,
+                                  near_id_tau2<T>(), false, o2));
+                const T *Ri2 = f32 ? (const T *)RinvT : (const T *)R2i;
                 EOD_CU((gemm<T, T, T, T>(false, false, m, p, p, 1.0, T1, m, Ri2, k, 0.0, Qb + kept * m, m, bup, &ws, s)));
-                EOD_CU(tdiag_product(R1, R2, k, pinf, tdiag_d + nt, s));
                 panel_p.push_back(p);
                 nt += p;
                 EOD_CU(oz_append(kept, p));
