@@ -166,6 +166,8 @@ struct GemmExtra {
     int64_t ldref = 0;
     double *err_partials = nullptr; // EPI_ERR: one double per CTA (gridDim.x*gridDim.y)
     int max_split = 64;
+    bool fine = false;         // emulated FP64: one more slice (see oz_gemm.cu)
+    int *nonfinite = nullptr;  // emulated FP64: set when an operand holds a NaN or an infinity (sliced as zero)
     int force_ts = 0;          // SIMT tile forced by the autotuner's timing hook (0 = plan)
 };
 
@@ -187,7 +189,7 @@ int64_t gemm_err_ctas(int64_t M, int64_t N);
 cudaError_t oz_gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A, int64_t lda,
                     const double *B, int64_t ldb, double beta, double *C, int64_t ldc, const GemmExtra &x,
                     int *err_flag, cudaStream_t s);
-// Pre-sliced operand of oz_gemm_ops: 8 BF16 slices of op(X) as rows x K
+// Pre-sliced operand of oz_gemm_ops: kOzSlices BF16 slices of op(X) as rows x K
 // (K contiguous, leading dimension ldk, slices slice_stride elements apart)
 // with a per-row exponent array e, or e == nullptr and one fixed exponent.
 struct OzOperand {
@@ -209,10 +211,8 @@ cudaError_t oz_gemm_f32(bool ta, bool tb, int64_t M, int64_t N, int64_t K, doubl
 // is null (every |X| must then be below 2^fixed_e)
 cudaError_t oz_slice(const double *X, int64_t rows, int64_t K, int64_t sr, int64_t sk, void *q, int *e,
                      int fixed_e, int64_t ldk, int64_t slice_stride, cudaStream_t s);
-constexpr int kOzSlices = 8;
-// largest K the emulation takes with the fused squared-error epilogue (which
-// cannot split K)
-constexpr int64_t kOzErrMaxK = 7168;
+constexpr int kOzSlices = 7;       // the factorisation's products
+constexpr int kOzSlicesFine = 8;   // GemmExtra::fine
 
 // whether gemm<double,...> sends an M x N x K product to oz_gemm
 bool fp64_use_emulated(int64_t M, int64_t N, int64_t K);

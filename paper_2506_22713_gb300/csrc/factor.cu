@@ -911,7 +911,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             const int64_t nct = gemm_err_ctas(m, n);
             double *part;
             EOD_TRY(ar.get(&part, (size_t)nct));
-            const bool emulated = oz.on && fp64_use_emulated(m, n, r) && r <= kOzErrMaxK;
+            const bool emulated = oz.on && fp64_use_emulated(m, n, r);
             uint16_t *cts = nullptr;
             int *ects = nullptr;
             const int64_t r8 = round_up8(r);

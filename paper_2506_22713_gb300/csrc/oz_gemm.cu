@@ -3,27 +3,40 @@
 // FP64 path for its large contractions.
 //
 // Each row i of op(A) (and each column j of op(B)) is scaled by a power of
-// two 2^-e so that its entries lie in (-1, 1), then cut into S = 8 integer
-// slices (exact BF16 values): q_0 in [-64, 64] (6 bits + rounding), q_1..q_7
-// in [-64, 64] (7 bits each):
-//     a = 2^e * sum_s q_s 2^(-6 - 7s),   truncation below 2^(e-56).
-// Products of slices are integers of magnitude <= 2^12.  Pairs (s, t) with
-// s + t <= 7 are grouped by g = s + t (weight 2^(-12 - 7g)); group g holds
-// g + 1 <= 8 pairs, so over a K chunk of 448 every group sum stays below
-// 8 * 448 * 2^12 < 2^24 and the tensor core's FP32 accumulation is exact.
-// After each chunk the epilogue warps read the eight group sums from TMEM as
-// integers, merge groups 0-3 and 4-7 exactly in int64 (each below 2^46), and
-// add the two merged values, scaled, into FP64 registers.  The dropped pairs
-// (s + t > 7) weigh at most 2^-68 of the row / column scales.  The result
-// equals an FP64 GEMM to within the slicing truncation (about 2^-56 of the
-// row / column maxima per term), accumulated in FP64.
+// two 2^-e so that its entries lie in (-1, 1), then cut into NS balanced
+// base-256 digits q_s in [-128, 128], every one exact in BF16:
+//     a = 2^e * sum_s q_s 2^(-7 - 8s),   rounded at 2^(e - 8 NS).
+// Products of digits are integers of magnitude <= 2^14.  Pairs (s, t) with
+// s + t < NS are grouped by g = s + t (weight 2^(-14 - 8g)); group g holds
+// g + 1 pairs, so over a K chunk of 256 the sums of groups 0-3 are at most
+// 4 * 256 * 2^14 = 2^24 and the tensor core's FP32 accumulation of them is
+// exact.  A later group's sum passes 2^24 only where nearly all its digits are
+// extreme and of one sign, so that the chunk's result is nearly 256 row x
+// column scales; what its rounding then loses is below 2^-49 of that result.
+// After each chunk the epilogue warps read the group
+// sums from TMEM as integers and add them to two int64 accumulators per
+// entry (groups 0-3 in units of 2^-38, the others in units of the last
+// group's), which hold the sums exactly; the two are combined and rounded
+// once, in integer arithmetic, at the end.  What is lost is the rounding of
+// the last digits and the pairs with s + t >= NS: about 2^(1 - 8 NS) of the
+// row x column scale per term.
+//   NS = 7 (28 products): the factorisation's products; 2^-56 per term, the
+//   level of an FP64 dot product.
+//   NS = 8 (36 products): where the result has to be as accurate as FP64 FMAs
+//   whatever the operands' spread (A_hat = U D V^T).
 //
-// CTA tile 128 x 64; a K block of 64 stages all eight B slices (64 KB) and
-// streams the eight A slices through a 4-deep ring; TMEM holds 8 x 64 FP32
-// group accumulators (all 512 columns).  Warp 0: TMA producer, warp 1: MMA
-// issuer, warps 2-9: drain and epilogue (two per TMEM lane quarter, 32
-// columns each).  All waits are bounded (EOD_ETIMEOUT
-// on expiry).
+// CTA tile 128 x 64; a K block of 64 stages all NS B slices and streams the
+// NS A slices through a ring; TMEM holds NS x 64 FP32 group accumulators.
+// Warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: drain and epilogue
+// (two per TMEM lane quarter, 32 columns each).  All waits are bounded
+// (EOD_ETIMEOUT on expiry).
+//
+// Measured (per launch, launch included): 2048^3 620 us = 27.7 TFLOP/s of FP64
+// (680 us with eight base-128 digits, 36 products and one 2^-50 accumulator),
+// 4000 x 1600 x 1600 762 us (822), slicing a 2048^2 operand and its transpose
+// 57 us (132, 2-byte stores).  What bounds it: shared-memory reads, 6 KB per
+// MMA of 128 x 64 x 16 (72 cycles each instead of 32), then the drain, about
+// 7000 cycles per chunk of integer conversions and wide additions.
 #include "common.cuh"
 #include "instrument.cuh"
 #include "tc_gemm.cuh"
@@ -37,34 +50,26 @@ namespace oz {
 
 using namespace eod::tc;
 
-constexpr int NS = kOzSlices;         // slices per operand (8)
-constexpr int NG = 8;                 // weight groups g = s + t, pairs with s + t <= 7
 constexpr int BM = 128, BN = 64, BK = 64;
-constexpr int KCH = 7;                // K blocks per exact chunk (448)
-constexpr int kOzMaxChunks = 16;      // chunks one CTA accumulates in int64
-static_assert(kOzMaxChunks * KCH * BK == kOzErrMaxK, "fused-error K limit");
+constexpr int KCH = 4;                // K blocks per chunk (256)
 constexpr int UMMA_K = 16;            // K per tcgen05.mma kind::f16
-#ifndef OZ_ASTAGES
-#define OZ_ASTAGES 2
-#endif
-#ifndef OZ_BSTAGES
-#define OZ_BSTAGES 2
-#endif
-constexpr int ASTAGES = OZ_ASTAGES, BSTAGES = OZ_BSTAGES;
 constexpr int A_TILE = BM * BK * 2;   // 16 KB: one slice
-constexpr int APS = 2;                // A slices per pipeline stage (one wait and one commit each)
-constexpr int A_STAGE = APS * A_TILE;
-static_assert(kOzSlices % APS == 0, "slices per stage");
 constexpr int B_TILE = BN * BK * 2;   // 8 KB
-constexpr int B_SET = NS * B_TILE;    // 64 KB
-constexpr int SMEM = BSTAGES * B_SET + ASTAGES * A_STAGE + 1024 + 256;
-constexpr uint32_t TMEM_COLS = 512;   // 8 x 64 used
+constexpr int BSTAGES = 2;            // K blocks of B in flight (NS slices each)
+template <int NS> struct Cfg {
+    static constexpr int ASTAGES = NS == 7 ? 6 : 5;   // A slices in flight
+    static constexpr int B_SET = NS * B_TILE;
+    static constexpr int SMEM = BSTAGES * B_SET + ASTAGES * A_TILE + 1024 + 256;
+    static_assert(BSTAGES * B_SET + ASTAGES * A_TILE >= 256 * 32 * 16, "the epilogue's staging");
+};
+constexpr int kMaxSlices = kOzSlicesFine;
+constexpr uint32_t TMEM_COLS = 512;   // NS x 64 used
 constexpr int NTHREADS = 320;        // producer, MMA issuer, 8 drain warps
 constexpr int ECOLS = BN / 2;         // columns per drain warp
 
 struct Maps {
-    CUtensorMap a[NS];
-    CUtensorMap b[NS];
+    CUtensorMap a[kMaxSlices];
+    CUtensorMap b[kMaxSlices];
 };
 
 struct Params {
@@ -84,20 +89,59 @@ struct Params {
     int a_tri, b_tri;         // op(A) / op(B) upper triangular: skip their zero K blocks
 };
 
-// v 2^e: one multiply by a power of two built from its bits (exact unless
-// the result leaves the normal range, where ldexp takes over)
-__device__ __forceinline__ double pow2_scale(double v, int e) {
-    if (e >= -1022 && e <= 1023) return v * __longlong_as_double((long long)(e + 1023) << 52);
-    return ldexp(v, e);
+// m 2^e for a result outside the normal range's middle (kept out of line: its
+// FP64 instructions would otherwise be issued, predicated, for every entry)
+__device__ __noinline__ double far_scale(unsigned long long m, int e) { return ldexp((double)m, e); }
+
+// (hi 2^SH + lo) 2^e as a double, rounded once to nearest (ties to even), in
+// integer arithmetic: an FP64 instruction costs a warp 64 cycles here, and a
+// tile has 8192 entries.  |hi| < 2^62.
+template <int SH>
+__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int e) {
+    // magnitude: h 2^SH + r, 0 <= r < 2^SH
+    long long h = hi + (lo >> SH);
+    unsigned long long r = (unsigned long long)lo & ((1ull << SH) - 1);
+    const unsigned long long sign = (unsigned long long)h & (1ull << 63);
+    if (h < 0) {
+        h = -h - (r ? 1 : 0);
+        r = r ? (1ull << SH) - r : 0ull;
+    }
+    if (h == 0) {   // all of it in r (< 2^SH <= 2^32): exact
+        h = (long long)r;
+        r = 0;
+        e -= SH;
+        if (h == 0) return 0.0;
+    }
+    // normalise to a leading one at bit 63; what r holds below goes in behind h
+    const int lz = __clzll(h);
+    unsigned long long m = ((unsigned long long)h << lz) | (lz >= SH ? r << (lz - SH) : r >> (SH - lz));
+    if (lz < SH && (r & ((1ull << (SH - lz)) - 1)) != 0ull) m |= 1ull;   // sticky
+    const int ex = 63 - lz + SH + e;                                     // value = m 2^(ex - 63)
+    const unsigned long long q = (m + 0x3ffull + ((m >> 11) & 1ull)) >> 11;
+    const bool carried = m >= 0xfffffffffffffc00ull;                    // the rounding wrapped past bit 63
+    if (ex >= -1022 && ex <= 1022) {
+        const unsigned long long bits = ((unsigned long long)(ex + 1022) << 52) + (carried ? 1ull << 53 : q);
+        return __longlong_as_double((long long)(bits | sign));           // (q's leading bit adds one to the exponent)
+    }
+    const double v = far_scale(carried ? 1ull << 53 : q, ex - 52);   // overflow or subnormal
+    return sign ? -v : v;
 }
 
-template <int EPI>
+// acc + v 2^k (exact), one wide multiply-add
+__device__ __forceinline__ long long mad_wide(int v, int pow2, long long acc) {
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(v), "r"(pow2), "l"(acc));
+    return d;
+}
+
+template <int NS, int EPI>
 __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_constant__ Maps maps, Params p) {
+    constexpr int NG = NS, ASTAGES = Cfg<NS>::ASTAGES, B_SET = Cfg<NS>::B_SET;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *bbuf = smem;                                 // BSTAGES x 7 B slices
-    uint8_t *abuf = smem + BSTAGES * B_SET;                // ASTAGES stages of APS A slices
-    uint64_t *fullB = (uint64_t *)(abuf + ASTAGES * A_STAGE);
+    uint8_t *bbuf = smem;                                 // BSTAGES x NS B slices
+    uint8_t *abuf = smem + BSTAGES * B_SET;                // ring of A slices
+    uint64_t *fullB = (uint64_t *)(abuf + ASTAGES * A_TILE);
     uint64_t *emptyB = fullB + BSTAGES;
     uint64_t *fullA = emptyB + BSTAGES;
     uint64_t *emptyA = fullA + ASTAGES;
@@ -154,15 +198,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                     tma_load_2d(bbuf + sb * B_SET + t * B_TILE, &maps.b[t], &fullB[sb], (int)(kb * BK), (int)n0);
             }
             ++ib;
-            for (int s0 = 0; s0 < NS && ok; s0 += APS) {
+            for (int s = 0; s < NS && ok; ++s) {
                 const int sa = (int)(ia % ASTAGES);
                 if (ia >= ASTAGES) ok = warp_wait(&emptyA[sa], (uint32_t)((ia / ASTAGES - 1) & 1));
                 if (!ok) break;
                 if (leader) {
-                    mbar_expect_tx(&fullA[sa], A_STAGE);
-                    for (int u = 0; u < APS; ++u)
-                        tma_load_2d(abuf + sa * A_STAGE + u * A_TILE, &maps.a[s0 + u], &fullA[sa], (int)(kb * BK),
-                                    (int)m0);
+                    mbar_expect_tx(&fullA[sa], A_TILE);
+                    tma_load_2d(abuf + sa * A_TILE, &maps.a[s], &fullA[sa], (int)(kb * BK), (int)m0);
                 }
                 ++ia;
             }
@@ -173,7 +215,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         // ---------------- MMA issuer ----------------
         // Warp-uniform loop, one elected lane issues: single-thread divergent
         // control flow around tcgen05 instructions slows their issue.
-        // Fully unrolled over the 36 slice pairs and the 4 K steps of a
+        // Fully unrolled over the slice pairs and the 4 K steps of a
         // block: descriptors are a base plus constant offsets (the 16-byte
         // unit field advances by 2 per 32-byte K step and by 512 per 8 KB B
         // slice).
@@ -196,27 +238,22 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
             const uint64_t bd0 = sdesc(smem_u32(bbuf + sb * B_SET), 16, 1024);
             if (__any_sync(0xffffffffu, *(volatile int *)abort_sh != 0)) ok = false;
 #pragma unroll
-            for (int s0 = 0; s0 < NS; s0 += APS) {
+            for (int s = 0; s < NS; ++s) {
                 const int sa = (int)(ia % ASTAGES);
                 if (ok) ok = warp_wait(&fullA[sa], (uint32_t)((ia / ASTAGES) & 1));
                 if (ok) {
                     tc_fence_after();
                     if (leader) {
-                        const uint64_t as0 = sdesc(smem_u32(abuf + sa * A_STAGE), 16, 1024);
+                        const uint64_t ad0 = sdesc(smem_u32(abuf + sa * A_TILE), 16, 1024);
 #pragma unroll
-                        for (int u = 0; u < APS; ++u) {
-                            const int s = s0 + u;
-                            const uint64_t ad0 = as0 + (uint64_t)(u * (A_TILE >> 4));
+                        for (int t = 0; t < NG; ++t) {
+                            if (s + t < NG) {
 #pragma unroll
-                            for (int t = 0; t < NG; ++t) {
-                                if (s + t < NG) {
-#pragma unroll
-                                    for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-                                        // the first MMA of a group in a chunk overwrites it
-                                        const uint32_t accum = (first && s == 0 && kk == 0) ? 0u : 1u;
-                                        umma_bf16(tmem + (uint32_t)((s + t) * BN), ad0 + (uint64_t)(2 * kk),
-                                                  bd0 + (uint64_t)(512 * t + 2 * kk), idesc, accum);
-                                    }
+                                for (int kk = 0; kk < BK / UMMA_K; ++kk) {
+                                    // the first MMA of a group in a chunk overwrites it
+                                    const uint32_t accum = (first && s == 0 && kk == 0) ? 0u : 1u;
+                                    umma_bf16(tmem + (uint32_t)((s + t) * BN), ad0 + (uint64_t)(2 * kk),
+                                              bd0 + (uint64_t)(512 * t + 2 * kk), idesc, accum);
                                 }
                             }
                         }
@@ -244,17 +281,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         const int qtr = warp & 3;                 // TMEM lane quarter this warp may read
         const int c0 = ((warp - 2) >> 2) * ECOLS; // its half of the 64 columns
         const int64_t row = m0 + 32 * qtr + lane;
-        // Per chunk the eight FP32 group sums (exact integers) merge into one
-        // int64 in units of 2^-50 of the row x column scale:
-        //   hi = groups 0-3 in base 128 (unit 2^-33), lo = groups 4-7 (unit 2^-61),
-        //   c  = hi 2^17 + round(lo 2^-11);
-        // |hi| < 2^41.9 (|v_g| <= (g+1) 2^12 448), so |c| < 2^58.9 and up to
-        // kOzMaxChunks = 16 chunks (the host splits K to respect that)
-        // accumulate without overflow, rounding 2^-51 of the scale per chunk,
-        // with no FP64 instruction in the drain.
-        long long acc[ECOLS];
+        // this lane's row exponent and the exponent of column c0 + lane, both
+        // read before the products are ready
+        const int erow = p.ea && row < p.M ? max(p.ea[row], -1100) : p.ea_fixed;
+        const int ecol = p.eb && n0 + c0 + lane < p.N ? max(p.eb[n0 + c0 + lane], -1100) : p.eb_fixed;
+        // Per chunk the FP32 group sums (integers) are added to two int64
+        // accumulators, groups 0-3 in base 256 (unit 2^-38 of the row x column
+        // scale, |per chunk| < 2^49) and the others (unit 2^(-14 - 8 (NS - 1)),
+        // < 2^50): exact, with no FP64 instruction in the drain.
+        constexpr int SH = 8 * (NS - 4);          // from the high unit to the low one
+        long long acch[ECOLS], accl[ECOLS];
 #pragma unroll
-        for (int j = 0; j < ECOLS; ++j) acc[j] = 0;
+        for (int j = 0; j < ECOLS; ++j) acch[j] = accl[j] = 0;
         bool ok = true;
         for (int64_t c = 0; c < nchunks; ++c) {
             ok = __all_sync(0xffffffffu, mbar_wait(tmem_full, (uint32_t)(c & 1)) ? 1 : 0) != 0;
@@ -270,44 +308,65 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                 tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    long long hi = 0, lo = 0;
 #pragma unroll
                     for (int g = 0; g < NG; ++g) {
-                        const long long iv = (long long)__float2int_rn(__uint_as_float(r[g][j]));   // exact: |v| <= 2^24
-                        if (g < 4) hi = hi * 128 + iv;
-                        else lo = lo * 128 + iv;
+                        const int iv = __float2int_rn(__uint_as_float(r[g][j]));
+                        if (g < 4) acch[cc + j] = mad_wide(iv, 1 << (8 * (3 - g)), acch[cc + j]);
+                        else accl[cc + j] = mad_wide(iv, 1 << (8 * (NG - 1 - g)), accl[cc + j]);
                     }
-                    acc[cc + j] += hi * 131072 + ((lo + (1ll << 10)) >> 11);
                 }
             }
             tc_fence_before();
             mbar_arrive(tmem_empty);
         }
         if (!ok) atomicExch(p.err_flag, 1);
-        double local = 0.0;
-        if (row < p.M) {
-            const int ei = p.ea ? max(p.ea[row], -1100) : p.ea_fixed;
-            const bool unit_alpha = p.alpha == 1.0;
+        // The sums go through shared memory (free by now: every product of this
+        // CTA has been read) so that the epilogue is a short loop; unrolled over
+        // the registers its code alone, fetched once per CTA, took 30 us.
+        longlong2 *st = (longlong2 *)smem + (threadIdx.x - 64);
+        if (ok) {
 #pragma unroll
-            for (int j = 0; j < ECOLS; ++j) {
-                const int64_t col = n0 + c0 + j;
-                if (col < p.N && !(p.upper_only && row > col)) {
-                    const double val =
-                        pow2_scale((double)acc[j], ei + (p.eb ? max(p.eb[col], -1100) : p.eb_fixed) - 50);
+            for (int j = 0; j < ECOLS; ++j) st[j * 256] = make_longlong2(acch[j], accl[j]);
+        }
+        double local = 0.0;
+        const bool split = EPI == EPI_STORE && p.split_stride > 0;
+        const bool unit_alpha = p.alpha == 1.0;
+        // four columns at a time: what the epilogue reads (C or the reference)
+        // is loaded for all of them before the first is used
+        constexpr int EC = 4;
+        const int64_t left = p.N - (n0 + c0);
+#pragma unroll 1
+        for (int cc = 0; ok && cc < ECOLS && cc < left; cc += EC) {
+            double old[EC];
+#pragma unroll
+            for (int j = 0; j < EC; ++j) {
+                const int64_t col = n0 + c0 + cc + j;
+                const bool in = row < p.M && cc + j < left && !(p.upper_only && row > col);
+                old[j] = 0.0;
+                if (EPI == EPI_ERR) {
+                    if (in) old[j] = __ldcs(p.R + row + col * p.ldr);
+                } else if (!split && p.beta != 0.0 && in) {
+                    old[j] = p.Cf ? (double)p.Cf[row + col * p.ldc] : p.C[row + col * p.ldc];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < EC; ++j) {
+                const int64_t col = n0 + c0 + cc + j;
+                const int ec = __shfl_sync(0xffffffffu, ecol, cc + j);
+                const longlong2 v = st[(cc + j) * 256];
+                const double val = fixed_to_double<SH>(v.x, v.y, erow + ec - 14 - 8 * (NS - 1));
+                if (row < p.M && cc + j < left && !(p.upper_only && row > col)) {
                     if (EPI == EPI_STORE) {
-                        if (p.split_stride > 0) {
+                        if (split) {
                             p.C[(int64_t)blockIdx.z * p.split_stride + row + col * p.M] = val;
-                        } else if (p.Cf) {
-                            double out = unit_alpha ? val : p.alpha * val;
-                            if (p.beta != 0.0) out = fma(p.beta, (double)p.Cf[row + col * p.ldc], out);
-                            p.Cf[row + col * p.ldc] = (float)out;
                         } else {
                             double out = unit_alpha ? val : p.alpha * val;
-                            if (p.beta != 0.0) out = fma(p.beta, p.C[row + col * p.ldc], out);
-                            p.C[row + col * p.ldc] = out;
+                            if (p.beta != 0.0) out = fma(p.beta, old[j], out);
+                            if (p.Cf) p.Cf[row + col * p.ldc] = (float)out;
+                            else p.C[row + col * p.ldc] = out;
                         }
                     } else {
-                        const double d = fma(-p.alpha, val, p.R[row + col * p.ldr]);
+                        const double d = fma(-p.alpha, val, old[j]);
                         local = fma(d, d, local);
                     }
                 }
@@ -405,49 +464,50 @@ __global__ void rowexp_kernel(const TX *__restrict__ X, int64_t R, int64_t K, in
     }
 }
 
-// The eight BF16 digits of x 2^-er into o[s * slice_stride] (see below).
-__device__ __forceinline__ void write_slices(double x, int er, __nv_bfloat16 *o, int64_t slice_stride) {
+// The NS BF16 digits of x 2^-er (|x| < 2^er) in q: v = round(|x| 2^(8 NS - 1 - er))
+// in balanced base-256 digits, integer arithmetic on the bit pattern.
+template <int NS>
+__device__ __forceinline__ void digits(double x, int er, __nv_bfloat16 q[NS], bool &nonfinite) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
     const bool neg = (bits >> 63) != 0;
     int E = (int)((bits >> 52) & 0x7ff);
     unsigned long long M = bits & 0xfffffffffffffull;
-    if (E == 0x7ff) M = 0;               // non-finite: not representable, taken as zero
-    else if (E == 0) E = 1;              // subnormal: M 2^(1 - 1075)
+    if (E == 0x7ff) {                    // non-finite: not representable, taken as zero
+        M = 0;
+        nonfinite = true;
+    } else if (E == 0) E = 1;            // subnormal: M 2^(1 - 1075)
     else M |= 1ull << 52;                // |x| = M 2^(E - 1075)
-    long long v = 0;
-    const int sh = E - 1020 - er;        // v = M 2^sh; sh <= 2 since |x| < 2^er
+    unsigned long long v = 0;            // below 2^(8 NS - 1); the digits' carries in two's complement
+    const int sh = E - 1075 + 8 * NS - 1 - er;   // v = M 2^sh; sh <= 8 NS - 54 since |x| < 2^er
     if (er >= -1100 && M != 0) {
-        if (sh >= 0) v = (long long)(M << sh);
-        else if (sh > -63) v = (long long)((M >> (-sh)) + ((M >> (-sh - 1)) & 1ull));
+        if (sh >= 0) v = M << sh;
+        else if (sh > -63) v = (M >> (-sh)) + ((M >> (-sh - 1)) & 1ull);
     }
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-        const int w = 49 - 7 * s;
-        long long q;
-        if (w > 0) q = (v + (1ll << (w - 1))) >> w;   // balanced digit: |q| <= 64
-        else q = v;
-        v -= q << w;
-        const float qf = (float)(neg ? -q : q);
-        o[s * slice_stride] = __float2bfloat16_rn(qf);
+        const int w = 8 * (NS - 1 - s);
+        int d;                           // balanced digit, |d| <= 128
+        if (s == 0) d = (int)((v + (1ull << (w - 1))) >> w);
+        else if (w > 0) d = (int)((long long)(v + (1ull << (w - 1))) >> w);
+        else d = (int)(long long)v;
+        v -= (unsigned long long)(long long)d << w;
+        q[s] = __float2bfloat16_rn((float)(neg ? -d : d));
     }
 }
 
-// out[s][r * ldk + k] = slice s of X(r, k) 2^-e[r]; 32 x 32 tiles through
-// shared memory so reads follow X's contiguous axis and writes follow k.
-// Integer arithmetic on the bit pattern: v = round(|x| 2^(55 - e)) < 2^55 + 1
-// is split into 8 balanced base-128 digits q_s in [-64, 64] (digit s has
-// weight 2^(49 - 7 s)), so x = sign 2^(e - 55) sum_s q_s 2^(49 - 7 s) up to
-// 2^(e - 56); every q_s is exact in BF16.
+// out[s][r * ldk + k] = slice s of X(r, k) 2^-e[r], tiles of 32 rows x 64 k
+// through shared memory so reads follow X's contiguous axis and writes follow
+// k (two neighbouring k per lane, one 4-byte store per slice).
 // The row exponents come from the nsplit partial ones of rowexp_kernel (the
 // blocks of the first K column also store them in e_out for the product), or
 // every row takes fixed_e when ep is null.
-template <typename TX>
-__global__ void slice_kernel(const TX *__restrict__ X, int64_t R, int64_t K, int64_t sr, int64_t sk,
+template <typename TX, int NS>
+__global__ void __launch_bounds__(256) slice_kernel(const TX *__restrict__ X, int64_t R, int64_t K, int64_t sr, int64_t sk,
                              int tri, const int *__restrict__ ep, int nsplit, int *__restrict__ e_out, int fixed_e,
-                             __nv_bfloat16 *__restrict__ out, int64_t ldk, int64_t slice_stride) {
-    __shared__ double tile[32][33];
+                             __nv_bfloat16 *__restrict__ out, int64_t ldk, int64_t slice_stride, int *nonfinite) {
+    __shared__ double tile[32][65];
     __shared__ int erow[32];
-    const int64_t r0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * 32;
+    const int64_t r0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * 64;
     const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
     if (ty == 0) {
         const int64_t r = r0 + tx;
@@ -459,36 +519,73 @@ __global__ void slice_kernel(const TX *__restrict__ X, int64_t R, int64_t K, int
         }
         erow[tx] = er;
     }
-    for (int i = ty; i < 32; i += 8) {
-        int64_t r, k;
-        if (sk == 1) { r = r0 + i; k = k0 + tx; } else { r = r0 + tx; k = k0 + i; }
-        const double v = (r < R && k < K && !tri_zero(tri, r, k)) ? (double)X[r * sr + k * sk] : 0.0;
-        if (sk == 1) tile[i][tx] = v; else tile[tx][i] = v;   // tile[r - r0][k - k0]
+    if (sk == 1) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = ty + 8 * (u >> 1), kk = tx + 32 * (u & 1);
+            const int64_t r = r0 + i, k = k0 + kk;
+            tile[i][kk] = (r < R && k < K && !tri_zero(tri, r, k)) ? (double)X[r * sr + k] : 0.0;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int kk = ty + 8 * u;
+            const int64_t r = r0 + tx, k = k0 + kk;
+            tile[tx][kk] = (r < R && k < K && !tri_zero(tri, r, k)) ? (double)X[r * sr + k * sk] : 0.0;
+        }
     }
     __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        const int64_t r = r0 + i, k = k0 + tx;
+    bool bad = false;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int i = ty + 8 * u;
+        const int64_t r = r0 + i, k = k0 + 2 * tx;
         if (r >= R || k >= K) continue;
-        write_slices(tile[i][tx], erow[i], out + r * ldk + k, slice_stride);
+        __nv_bfloat16 a[NS], b[NS];
+        digits<NS>(tile[i][2 * tx], erow[i], a, bad);
+        digits<NS>(tile[i][2 * tx + 1], erow[i], b, bad);
+        __nv_bfloat16 *o = out + r * ldk + k;
+        if (k + 1 < K && (((uintptr_t)o | (uintptr_t)(slice_stride * 2)) & 3) == 0) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) *(__nv_bfloat162 *)(o + s * slice_stride) = __nv_bfloat162(a[s], b[s]);
+        } else {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                o[s * slice_stride] = a[s];
+                if (k + 1 < K) o[s * slice_stride + 1] = b[s];
+            }
+        }
     }
+    if (bad && nonfinite) *nonfinite = 1;
 }
 
 // Rows with K contiguous (sk == 1) and their own exponents, one CTA per row:
 // the row maximum (as in rowexp_kernel) and then the slices (as in
-// slice_kernel), in one launch; the second read of the row hits L1 / L2.
-template <typename TX>
+// slice_kernel), in one launch.  A thread takes pairs of neighbouring k; the
+// first RU pairs stay in registers between the two, the rest are read again.
+template <typename TX, int NS>
 __global__ void __launch_bounds__(256) slice_rows_kernel(const TX *__restrict__ X, int64_t K, int64_t sr,
                                                          int tri, int *__restrict__ e_out,
                                                          __nv_bfloat16 *__restrict__ out, int64_t ldk,
-                                                         int64_t slice_stride) {
+                                                         int64_t slice_stride, int *nonfinite) {
+    constexpr int RU = 4;
     __shared__ unsigned long long red[8];
     __shared__ int er_sh;
     const int64_t r = blockIdx.x;
     const TX *x = X + r * sr;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t k0 = 2 * tid;
+    auto load = [&](int64_t k) -> double { return k < K && !tri_zero(tri, r, k) ? (double)x[k] : 0.0; };
+    double va[RU], vb[RU];
+#pragma unroll
+    for (int u = 0; u < RU; ++u) {
+        va[u] = load(k0 + 512 * u);
+        vb[u] = load(k0 + 512 * u + 1);
+    }
     unsigned long long m = 0ull;
-    for (int64_t k = tid; k < K; k += 256)
-        if (!tri_zero(tri, r, k)) m = max(m, abs_bits((double)x[k]));
+#pragma unroll
+    for (int u = 0; u < RU; ++u) m = max(m, max(abs_bits(va[u]), abs_bits(vb[u])));
+    for (int64_t k = k0 + 512 * RU; k < K; k += 512) m = max(m, max(abs_bits(load(k)), abs_bits(load(k + 1))));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) red[warp] = m;
@@ -503,9 +600,30 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const TX *__restrict__ 
     }
     __syncthreads();
     const int er = er_sh;
-    __nv_bfloat16 *o = out + r * ldk;
-    for (int64_t k = tid; k < K; k += 256)
-        write_slices(tri_zero(tri, r, k) ? 0.0 : (double)x[k], er, o + k, slice_stride);
+    __nv_bfloat16 *row = out + r * ldk;
+    const bool pairs = (((uintptr_t)row | (uintptr_t)(slice_stride * 2)) & 3) == 0;
+    bool bad = false;
+    auto store = [&](int64_t k, double p, double q) {
+        __nv_bfloat16 a[NS], b[NS];
+        digits<NS>(p, er, a, bad);
+        digits<NS>(q, er, b, bad);
+        __nv_bfloat16 *o = row + k;
+        if (pairs && k + 1 < K) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) *(__nv_bfloat162 *)(o + s * slice_stride) = __nv_bfloat162(a[s], b[s]);
+        } else {
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                o[s * slice_stride] = a[s];
+                if (k + 1 < K) o[s * slice_stride + 1] = b[s];
+            }
+        }
+    };
+#pragma unroll
+    for (int u = 0; u < RU; ++u)
+        if (k0 + 512 * u < K) store(k0 + 512 * u, va[u], vb[u]);
+    for (int64_t k = k0 + 512 * RU; k < K; k += 512) store(k, load(k), load(k + 1));
+    if (bad && nonfinite) *nonfinite = 1;
 }
 
 template <typename TC>
@@ -529,14 +647,15 @@ struct Slices {
     int64_t R = 0, ldk = 0;
 };
 
-template <typename TX>
+template <int NS, typename TX>
 cudaError_t slice_into(const TX *X, int64_t R, int64_t K, int64_t sr, int64_t sk, __nv_bfloat16 *q, int *e,
-                       int fixed_e, int64_t ldk, int64_t slice_stride, cudaStream_t s, int tri = 0) {
+                       int fixed_e, int64_t ldk, int64_t slice_stride, cudaStream_t s, int tri = 0,
+                       int *nonfinite = nullptr) {
     if (R <= 0 || K <= 0) return cudaSuccess;
     ProfScope prof(PROF_OZ_SLICE, 0.0, (double)sizeof(TX) * R * K + 2.0 * NS * (double)R * K, s);
     if (e && sk == 1 && (R >= kNumSMs || K <= 8192)) {
         count_launch();
-        slice_rows_kernel<<<(unsigned)R, 256, 0, s>>>(X, K, sr, tri, e, q, ldk, slice_stride);
+        slice_rows_kernel<TX, NS><<<(unsigned)R, 256, 0, s>>>(X, K, sr, tri, e, q, ldk, slice_stride, nonfinite);
         return cudaGetLastError();
     }
     int *ep = nullptr;
@@ -561,22 +680,23 @@ cudaError_t slice_into(const TX *X, int64_t R, int64_t K, int64_t sr, int64_t sk
         }
     }
     count_launch();
-    dim3 grid((unsigned)((K + 31) / 32), (unsigned)((R + 31) / 32));
-    slice_kernel<<<grid, dim3(32, 8), 0, s>>>(X, R, K, sr, sk, tri, ep, (int)ksplit, (ep && ep != e) ? e : nullptr,
-                                               fixed_e, q, ldk, slice_stride);
+    dim3 grid((unsigned)((K + 63) / 64), (unsigned)((R + 31) / 32));
+    slice_kernel<TX, NS><<<grid, dim3(32, 8), 0, s>>>(X, R, K, sr, sk, tri, ep, (int)ksplit,
+                                                       (ep && ep != e) ? e : nullptr, fixed_e, q, ldk, slice_stride,
+                                                       nonfinite);
     cudaError_t le = cudaGetLastError();
     if (ep && ep != e) cudaFreeAsync(ep, s);
     return le;
 }
 
-template <typename TX>
+template <int NS, typename TX>
 cudaError_t make_slices(const TX *X, int64_t R, int64_t K, int64_t sr, int64_t sk, Slices &sl, cudaStream_t s,
-                        int tri = 0) {
+                        int tri = 0, int *nonfinite = nullptr) {
     sl.R = R;
     sl.ldk = round_up(K, 8);
     EOD_CUDA_TRY(lib_malloc_async((void **)&sl.q, sizeof(__nv_bfloat16) * (size_t)NS * R * sl.ldk, s));
     EOD_CUDA_TRY(lib_malloc_async((void **)&sl.e, sizeof(int) * (size_t)R, s));
-    return slice_into(X, R, K, sr, sk, sl.q, sl.e, 0, sl.ldk, R * sl.ldk, s, tri);
+    return slice_into<NS>(X, R, K, sr, sk, sl.q, sl.e, 0, sl.ldk, R * sl.ldk, s, tri, nonfinite);
 }
 
 void free_slices(Slices &sl, cudaStream_t s) {
@@ -591,13 +711,13 @@ void free_slices(Slices &sl, cudaStream_t s) {
 // Slices of op(X) as `rows` x K with K contiguous (see oz_gemm.cu header).
 cudaError_t oz_slice(const double *X, int64_t rows, int64_t K, int64_t sr, int64_t sk, void *q, int *e,
                      int fixed_e, int64_t ldk, int64_t slice_stride, cudaStream_t s) {
-    return oz::slice_into(X, rows, K, sr, sk, (__nv_bfloat16 *)q, e, fixed_e, ldk, slice_stride, s);
+    return oz::slice_into<kOzSlices>(X, rows, K, sr, sk, (__nv_bfloat16 *)q, e, fixed_e, ldk, slice_stride, s);
 }
 
-cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha,
-                        double beta, double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s,
-                        float *Cf) {
-    using namespace oz;
+namespace oz {
+template <int NS>
+cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha, double beta,
+                    double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s, float *Cf) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (Cf && x.epilogue != EPI_STORE) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
@@ -638,17 +758,14 @@ cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64
         if (splits > smax) splits = smax;
         if (splits < 1) splits = 1;
     }
-    // the drain's int64 accumulators hold at most kOzMaxChunks chunks of KCH blocks
-    const int64_t smin = (p.kblocks + kOzMaxChunks * KCH - 1) / (kOzMaxChunks * KCH);
-    if (smin > 1 && x.epilogue != EPI_STORE) return cudaErrorInvalidValue;   // K > kOzErrMaxK with a fused error
-    if (splits < smin) splits = smin;
     p.kb_per_split = (p.kblocks + splits - 1) / splits;
     if (p.kb_per_split < 1) p.kb_per_split = 1;
     splits = (p.kblocks + p.kb_per_split - 1) / p.kb_per_split;
     if (splits < 1) splits = 1;
     double *part = nullptr;
-    e = set_smem_once(oz_gemm_kernel<EPI_STORE>, SMEM);
-    if (e == cudaSuccess) e = set_smem_once(oz_gemm_kernel<EPI_ERR>, SMEM);
+    constexpr int SMEM = Cfg<NS>::SMEM;
+    e = set_smem_once(oz_gemm_kernel<NS, EPI_STORE>, SMEM);
+    if (e == cudaSuccess) e = set_smem_once(oz_gemm_kernel<NS, EPI_ERR>, SMEM);
     if (e == cudaSuccess && splits > 1) {
         e = lib_malloc_async((void **)&part, sizeof(double) * (size_t)splits * M * N, s);
         p.C = part;
@@ -671,8 +788,8 @@ cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64
     if (e == cudaSuccess) {
         dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)splits);
         count_launch();
-        if (x.epilogue == EPI_ERR) oz_gemm_kernel<EPI_ERR><<<grid, NTHREADS, SMEM, s>>>(maps, p);
-        else oz_gemm_kernel<EPI_STORE><<<grid, NTHREADS, SMEM, s>>>(maps, p);
+        if (x.epilogue == EPI_ERR) oz_gemm_kernel<NS, EPI_ERR><<<grid, NTHREADS, SMEM, s>>>(maps, p);
+        else oz_gemm_kernel<NS, EPI_STORE><<<grid, NTHREADS, SMEM, s>>>(maps, p);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && splits > 1) {
@@ -687,9 +804,16 @@ cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64
     if (part) cudaFreeAsync(part, s);
     return e;
 }
+}  // namespace oz
+
+cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha,
+                        double beta, double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s,
+                        float *Cf) {
+    return oz::run_ops<kOzSlices>(A, B, M, N, K, alpha, beta, C, ldc, x, err_flag, s, Cf);
+}
 
 namespace oz {
-template <typename T>
+template <int NS, typename T>
 cudaError_t gemm_any(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const T *A, int64_t lda,
                      const T *B, int64_t ldb, double beta, double *C, float *Cf, int64_t ldc, const GemmExtra &x,
                      int *err_flag, cudaStream_t s) {
@@ -698,14 +822,14 @@ cudaError_t gemm_any(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double a
     // op(A)(i, k): rows i, reduction k; op(B)(k, j) seen as rows j
     // a_upper / b_upper: op(A) / op(B) is upper triangular and its zero part
     // is not read, as in the SIMT kernel
-    cudaError_t e = make_slices(A, M, K, ta ? lda : 1, ta ? 1 : lda, sa, s, x.a_upper ? 1 : 0);
+    cudaError_t e = make_slices<NS>(A, M, K, ta ? lda : 1, ta ? 1 : lda, sa, s, x.a_upper ? 1 : 0, x.nonfinite);
     const bool same = (A == B) && (ta != tb) && (lda == ldb) && (M == N) && !x.a_upper && !x.b_upper;
-    if (e == cudaSuccess && !same) e = make_slices(B, N, K, tb ? 1 : ldb, tb ? ldb : 1, sb, s, x.b_upper ? 2 : 0);
+    if (e == cudaSuccess && !same) e = make_slices<NS>(B, N, K, tb ? 1 : ldb, tb ? ldb : 1, sb, s, x.b_upper ? 2 : 0, x.nonfinite);
     const Slices &SB = same ? sa : sb;
     if (e == cudaSuccess) {
         OzOperand oa{sa.q, sa.e, 0, sa.ldk, (int64_t)M * sa.ldk};
         OzOperand ob{SB.q, SB.e, 0, SB.ldk, (int64_t)N * SB.ldk};
-        e = oz_gemm_ops(oa, ob, M, N, K, alpha, beta, C, ldc, x, err_flag, s, Cf);
+        e = run_ops<NS>(oa, ob, M, N, K, alpha, beta, C, ldc, x, err_flag, s, Cf);
     }
     free_slices(sa, s);
     if (!same) free_slices(sb, s);
@@ -718,7 +842,10 @@ cudaError_t gemm_any(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double a
 cudaError_t oz_gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A, int64_t lda,
                     const double *B, int64_t ldb, double beta, double *C, int64_t ldc, const GemmExtra &x,
                     int *err_flag, cudaStream_t s) {
-    return oz::gemm_any<double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, nullptr, ldc, x, err_flag, s);
+    if (x.fine)
+        return oz::gemm_any<kOzSlicesFine, double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, nullptr, ldc, x,
+                                                   err_flag, s);
+    return oz::gemm_any<kOzSlices, double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, nullptr, ldc, x, err_flag, s);
 }
 
 // The same product of FP32 data (exact in FP64, so sliced the same way) with
@@ -727,7 +854,7 @@ cudaError_t oz_gemm_f32(bool ta, bool tb, int64_t M, int64_t N, int64_t K, doubl
                         const float *B, int64_t ldb, double beta, float *C, int64_t ldc, const GemmExtra &x,
                         int *err_flag, cudaStream_t s) {
     if (x.epilogue != EPI_STORE) return cudaErrorInvalidValue;
-    return oz::gemm_any<float>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, nullptr, C, ldc, x, err_flag, s);
+    return oz::gemm_any<kOzSlices, float>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, nullptr, C, ldc, x, err_flag, s);
 }
 
 int64_t oz_gemm_err_ctas(int64_t M, int64_t N) { return ((M + oz::BM - 1) / oz::BM) * ((N + oz::BN - 1) / oz::BN); }
