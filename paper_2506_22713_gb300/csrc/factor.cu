@@ -1125,8 +1125,37 @@ static eod_status reconstruct_impl(const eod_factors *f, T *Ahat, int64_t ld, cu
     GemmExtra ex, bu;
     bu.b_upper = true;
     const T *U = (const T *)f->U, *V = (const T *)f->V;
-    EOD_CU((gemm<T, T, T, T>(false, false, m, r, r, 1.0, U, m, Dt, r, 0.0, W, m, bu, &ws, s)));     // W = U D
-    EOD_CU((gemm<T, T, T, T>(false, true, m, n, r, 1.0, W, m, V, n, 0.0, Ahat, ld, ex, &ws, s)));  // A_hat = W V^T
+    auto products = [&]() -> cudaError_t {
+        const cudaError_t e = gemm<T, T, T, T>(false, false, m, r, r, 1.0, U, m, Dt, r, 0.0, W, m, bu, &ws, s);   // W = U D
+        return e != cudaSuccess ? e : gemm<T, T, T, T>(false, true, m, n, r, 1.0, W, m, V, n, 0.0, Ahat, ld, ex, &ws, s);
+    };
+    if (std::is_same<T, double>::value && fp64_use_emulated(m, n, r)) {
+        // FP64: the larger of the two products (or both) on the tensor cores,
+        // as in the factorisation.  The emulation takes non-finite entries for
+        // zero, and it needs room for the operands' slices: where either
+        // happens, the DFMA products below give the result instead.
+        int *flags;   // [0] a wait ran out, [1] a non-finite entry was sliced
+        EOD_TRY(ar.get(&flags, 2));
+        EOD_CU(cudaMemsetAsync(flags, 0, sizeof(int) * 2, s));
+        ws.err_flag = flags;
+        ex.nonfinite = bu.nonfinite = flags + 1;
+        ex.fine = bu.fine = true;
+        const cudaError_t e = products();
+        ws.err_flag = nullptr;
+        ex.nonfinite = bu.nonfinite = nullptr;
+        if (e == cudaSuccess) {
+            int h[2] = {0, 0};
+            EOD_CU(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s));
+            EOD_CU(cudaStreamSynchronize(s));
+            if (h[0]) return EOD_ETIMEOUT;
+            if (!h[1]) return EOD_OK;
+        } else if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+        } else {
+            return cuda_status(e);
+        }
+    }
+    EOD_CU(products());
     return EOD_OK;
 }
 
