@@ -246,7 +246,7 @@ class _DevArray:
     """A device buffer owned by an eod_factors struct, exposed to torch."""
 
     def __init__(self, ptr, rows, cols, ld, dtype, owner):
-        es = torch.empty((), dtype=dtype).element_size()
+        es = 8 if dtype == torch.float64 else 4
         self._owner = owner
         self.__cuda_array_interface__ = {
             "shape": (rows, cols),
@@ -270,7 +270,7 @@ class Factors:
         self.precision = f.precision
         self.rel_err, self.norm_a, self.eps, self.t_margin = f.rel_err, f.norm_a, f.eps, f.t_margin
         self.blocks, self.restarts, self.block_k = f.blocks, f.restarts, f.block_k
-        self.tdiag = [f.tdiag[i] for i in range(f.ntdiag)]
+        self.tdiag = f.tdiag[:f.ntdiag]
 
     def _view(self, name, rows, cols, ld, dtype):
         ptr = getattr(self._ptr.contents, name)

@@ -27,6 +27,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <atomic>
+#include <mutex>
 #include <thread>
 #include <vector>
 
@@ -52,20 +53,72 @@ static eod_status cuda_status(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? EOD_ENOMEM : EOD_ECUDA;
 }
 
+// Pinned 64-byte blocks for the host mirrors below, kept between calls: one
+// cudaMallocHost + cudaFreeHost pair takes about 280 us, a quarter of a small
+// factorisation.  A block belongs to one call at a time; at most kMost stay.
+class PinnedBlocks {
+public:
+    void *take() {
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            if (!free_.empty()) {
+                void *p = free_.back();
+                free_.pop_back();
+                return p;
+            }
+        }
+        void *p = nullptr;
+        if (cudaHostAlloc(&p, 64, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return p;
+    }
+    void give(void *p) {
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            if (free_.size() < kMost) {
+                free_.push_back(p);
+                return;
+            }
+        }
+        cudaFreeHost(p);
+    }
+
+private:
+    static constexpr size_t kMost = 64;   // as many as the batched form has worker streams at most
+    std::mutex mu_;
+    std::vector<void *> free_;
+};
+static PinnedBlocks &pinned_blocks() {
+    static PinnedBlocks *b = new PinnedBlocks;   // lives as long as the process: calls may come from exiting threads
+    return *b;
+}
+
 // Pinned host mirror of the small device results read once per decision.
 struct HostMirror {
     int *info = nullptr;      // [2]
     double *val = nullptr;    // [4]
     int *flag = nullptr;      // [1]
+    cudaStream_t s;
+    explicit HostMirror(cudaStream_t st) : s(st) {}
+    HostMirror(const HostMirror &) = delete;
+    HostMirror &operator=(const HostMirror &) = delete;
     eod_status init() {
-        void *p = nullptr;
-        if (cudaMallocHost(&p, 64) != cudaSuccess) { cudaGetLastError(); return EOD_ENOMEM; }
+        void *p = pinned_blocks().take();
+        if (!p) return EOD_ENOMEM;
         info = (int *)p;
         flag = info + 2;
         val = (double *)((char *)p + 16);
         return EOD_OK;
     }
-    ~HostMirror() { if (info) cudaFreeHost(info); }
+    // the block goes to another call only once no copy of this one can write it
+    // (a call that ends with an error may have some queued)
+    ~HostMirror() {
+        if (!info) return;
+        if (cudaStreamSynchronize(s) == cudaSuccess) pinned_blocks().give(info);
+        else cudaGetLastError();   // the context is lost: the block stays with it
+    }
 };
 
 inline int64_t round_up8(int64_t x) { return (x + 7) / 8 * 8; }
@@ -459,7 +512,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     if (k > cap) k = cap;
     const bool mixed = (o.precision == EOD_MIXED_BF16 || o.precision == EOD_MIXED_TF32);
 
-    HostMirror hm;
+    HostMirror hm(s);
     EOD_TRY(hm.init());
 
     // ---- workspace ----
