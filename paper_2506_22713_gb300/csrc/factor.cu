@@ -53,7 +53,7 @@ static eod_status cuda_status(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? EOD_ENOMEM : EOD_ECUDA;
 }
 
-// Pinned 64-byte blocks for the host mirrors below, kept between calls: one
+// Pinned 128-byte blocks for the host mirrors below, kept between calls: one
 // cudaMallocHost + cudaFreeHost pair takes about 280 us, a quarter of a small
 // factorisation.  A block belongs to one call at a time; at most kMost stay.
 class PinnedBlocks {
@@ -68,7 +68,7 @@ public:
             }
         }
         void *p = nullptr;
-        if (cudaHostAlloc(&p, 64, cudaHostAllocPortable) != cudaSuccess) {
+        if (cudaHostAlloc(&p, 128, cudaHostAllocPortable) != cudaSuccess) {
             cudaGetLastError();
             return nullptr;
         }
@@ -99,7 +99,8 @@ static PinnedBlocks &pinned_blocks() {
 struct HostMirror {
     int *info = nullptr;      // [2]
     double *val = nullptr;    // [4]
-    int *flag = nullptr;      // [1]
+    int *flag = nullptr;      // [2]
+    int *core = nullptr;      // [8]
     cudaStream_t s;
     explicit HostMirror(cudaStream_t st) : s(st) {}
     HostMirror(const HostMirror &) = delete;
@@ -110,6 +111,7 @@ struct HostMirror {
         info = (int *)p;
         flag = info + 2;
         val = (double *)((char *)p + 16);
+        core = (int *)((char *)p + 64);
         return EOD_OK;
     }
     // the block goes to another call only once no copy of this one can write it
@@ -429,6 +431,46 @@ static eod_status cholqr2(CoreWork<T> &w, T *W, int64_t rows, int64_t ldw, int64
         }
     }
     return EOD_OK;
+}
+
+// CholQR2 of at most 128 columns without a host read: W_in (rows x p, ld
+// rows; may be W) = W R with R into Rout (p x p, ld p), one leaf of width p per
+// pass, the second taking the first-order factor of a near-identity Gram by
+// itself.  info[0..3] receives (columns factored, code) of the two leaves: the
+// caller checks both later, and repeats with cholqr2 (the shifted passes) if
+// the first did not factor every column.
+template <typename T>
+static eod_status cholqr2_one_leaf(CoreWork<T> &w, const T *W_in, T *W, int64_t rows, int64_t p, double *Rout, int *info,
+                                   Scratch *ws, cudaStream_t s) {
+    constexpr bool f32 = std::is_same<T, float>::value;
+    GemmExtra bup, tri;
+    bup.b_upper = true;
+    tri.a_upper = tri.b_upper = true;
+    CholOut o;
+    if (f32) o.RinvF = (float *)w.InvT, o.ldf = kPB;
+    const T *Ri = f32 ? (const T *)w.InvT : (const T *)w.RiD;
+    double *Rd = f32 ? nullptr : w.RiD;
+    for (int pass = 0; pass < 2; ++pass) {
+        const T *src = pass == 0 ? W_in : w.Tmp;
+        T *dst = pass == 0 ? w.Tmp : W;
+        EOD_CU(gram_skinny<T>(src, rows, (int)p, rows, w.G, p, ws, s));
+        EOD_CU(chol_small(w.G, p, (int)p, 0, 0.0, 0.0, 0.0, 0.0, pass == 0 ? w.R : w.Rp, p, Rd, kPB, info + 2 * pass, s,
+                          pass == 0 ? 0.0 : near_id_tau2<T>(), false, o));
+        EOD_CU((gemm<T, T, T, T>(false, false, rows, p, p, 1.0, src, rows, Ri, kPB, 0.0, dst, rows, bup, ws, s)));
+    }
+    EOD_CU((gemm<double, double, double, double>(false, false, p, p, p, 1.0, w.Rp, p, w.R, p, 0.0, Rout, p, tri, ws, s)));
+    return EOD_OK;
+}
+
+// Whether the core's CholQR2 of an r-column factor takes one leaf per pass:
+// up to the leaf's widest, unless the table asks for narrower ones.
+// Whole calls, blocked form against one leaf per pass (which also drops the
+// fills, copies and host reads of the blocked form): 512 x 384 FP64, r = 20,
+// 705 -> 578 us; 262144 x 224 mixed, r = 13, 2040 -> 1740 us; n = 1000 FP64,
+// r = 104, 1881 -> 1828 us.
+static bool core_one_leaf(int64_t r) {
+    int64_t v = 0;
+    return r <= 128 && !(tuned_value("core_leaf", r, 0, 0, &v) && v < r);
 }
 
 // A non-blocking stream of the calling thread on the current device, for
@@ -844,34 +886,42 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
         }
     }
     if (ahead) EOD_CU(stream_after(s, s2));   // an unused lookahead: its buffers are shared after this
-    // the T diagonal recorded on the device, and every panel's second pass
-    // checked: it factored all p columns
-    if (nt > 0 || !panel_p.empty()) {
-        std::vector<int> pinf(2 * panel_p.size() + 1);
-        tdiag.resize((size_t)nt);
-        if (nt > 0) EOD_CU(cudaMemcpyAsync(tdiag.data(), tdiag_d, sizeof(double) * nt, cudaMemcpyDeviceToHost, s));
-        if (!panel_p.empty())
-            EOD_CU(cudaMemcpyAsync(pinf.data(), pinfo, sizeof(int) * 2 * panel_p.size(), cudaMemcpyDeviceToHost, s));
-        EOD_CU(cudaStreamSynchronize(s));
-        for (size_t i = 0; i < panel_p.size(); ++i)
-            if (pinf[2 * i] != panel_p[i] || pinf[2 * i + 1] != CHOL_ALL) return EOD_EPRECISION;
-    }
     const int64_t r = kept;
     F->rank = r;
     F->blocks = blocks;
     F->restarts = restarts;
 
-    // t_margin over the tested entries
-    double margin = INFINITY;
-    for (size_t i = 0; i < tdiag.size(); ++i)
-        if (tdiag[i] > 0.0 && eps > 0.0) margin = std::min(margin, std::fabs(std::log10(tdiag[i] / eps)));
-    F->t_margin = margin;
-    F->ntdiag = (int64_t)tdiag.size();
-    F->tdiag = (double *)std::malloc(sizeof(double) * std::max<size_t>(tdiag.size(), 1));
-    if (!F->tdiag) return EOD_ENOMEM;
-    if (!tdiag.empty()) std::memcpy(F->tdiag, tdiag.data(), sizeof(double) * tdiag.size());
+    // The T diagonal recorded on the device and every panel's second pass
+    // (which has to have factored all its columns) are read once, at the end:
+    // queue_tdiag queues the copies, finish_tdiag uses them once `s` is idle.
+    std::vector<int> pinf(2 * panel_p.size() + 1);
+    auto queue_tdiag = [&]() -> cudaError_t {
+        tdiag.resize((size_t)std::max<int64_t>(nt, (int64_t)tdiag.size()));
+        cudaError_t e = cudaSuccess;
+        if (nt > 0) e = cudaMemcpyAsync(tdiag.data(), tdiag_d, sizeof(double) * nt, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess && !panel_p.empty())
+            e = cudaMemcpyAsync(pinf.data(), pinfo, sizeof(int) * 2 * panel_p.size(), cudaMemcpyDeviceToHost, s);
+        return e;
+    };
+    auto finish_tdiag = [&]() -> eod_status {
+        for (size_t i = 0; i < panel_p.size(); ++i)
+            if (pinf[2 * i] != panel_p[i] || pinf[2 * i + 1] != CHOL_ALL) return EOD_EPRECISION;
+        // t_margin over the tested entries
+        double margin = INFINITY;
+        for (size_t i = 0; i < tdiag.size(); ++i)
+            if (tdiag[i] > 0.0 && eps > 0.0) margin = std::min(margin, std::fabs(std::log10(tdiag[i] / eps)));
+        F->t_margin = margin;
+        F->ntdiag = (int64_t)tdiag.size();
+        F->tdiag = (double *)std::malloc(sizeof(double) * std::max<size_t>(tdiag.size(), 1));
+        if (!F->tdiag) return EOD_ENOMEM;
+        if (!tdiag.empty()) std::memcpy(F->tdiag, tdiag.data(), sizeof(double) * tdiag.size());
+        return EOD_OK;
+    };
 
     if (r == 0) {
+        EOD_CU(queue_tdiag());
+        EOD_CU(cudaStreamSynchronize(s));
+        EOD_TRY(finish_tdiag());
         F->rel_err = (norm_a > 0.0) ? 1.0 : 0.0;
         if (!o.compute_err) F->rel_err = -1.0;
         return EOD_OK;
@@ -886,6 +936,10 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     EOD_TRY(ar.get(&Rt, (size_t)r * r));
     EOD_TRY(ar.get(&D, (size_t)r * r));
     EOD_TRY(ar.get(&Rc, (size_t)r * r));
+    T *Qh;          // the second QR's orthonormal factor
+    int *core_info; // (columns, code) of the core's leaves
+    EOD_TRY(ar.get(&Qh, (size_t)r * r));
+    EOD_TRY(ar.get(&core_info, 8));
     // work space of the CholQR passes (subspace iteration and core)
     CoreWork<T> cw;
     cw.pcap = r;
@@ -998,61 +1052,94 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
 
     // ---- steps 9-11 ----
     Phase ph_core("eod.core");
-    EOD_CU((copy_matrix<T, T>(Ct, n, V, n, n, r, false, s)));
-    EOD_TRY(cholqr2(cw, V, n, n, r, Rc, hm, &ws, s));                 // C^T = V R
-    EOD_CU((copy_matrix<double, T>(Rc, r, Rt, r, r, r, true, s)));    // R^T
-    EOD_TRY(cholqr2(cw, Rt, r, r, r, D, hm, &ws, s));                 // R^T = Qh D
-    if (oz.on && fp64_use_emulated(m, r, r)) {   // U = Q Qh
-        const int64_t r8 = round_up8(r);
-        uint16_t *qhs;
-        int *eqh;
-        EOD_TRY(ar.get(&qhs, (size_t)kOzSlices * r * r8));
-        EOD_TRY(ar.get(&eqh, (size_t)r));
-        EOD_CU(oz_slice((const double *)Rt, r, r, r, 1, qhs, eqh, 0, r8, r * r8, s));
-        const OzOperand qr{oz.Qr, nullptr, 1, oz.cap8, m * oz.cap8};
-        const OzOperand qho{qhs, eqh, 0, r8, r * r8};
-        EOD_CU(oz_gemm_ops(qr, qho, m, r, r, 1.0, 0.0, (double *)U, m, ex, ws.err_flag, s));
-    } else if (mixed && std::is_same<T, float>::value && m >= kTfMinRows && r >= 32) {
-        // U = Q Qh on the tensor cores as three TF32 products of split
-        // operands, X = X_hi + X_lo (X_hi Y_hi + X_hi Y_lo + X_lo Y_hi: about
-        // 2^-21 relative, the accuracy of an FP32 product); TF32 operands are
-        // K-major, so Q is split transposed (r4 x m)
-        const int64_t r4 = round_up(r, 4);
-        float *q_hi, *q_lo, *h_hi, *h_lo;
-        EOD_TRY(ar.get(&q_hi, (size_t)(r4 * m)));
-        EOD_TRY(ar.get(&q_lo, (size_t)(r4 * m)));
-        EOD_TRY(ar.get(&h_hi, (size_t)(r4 * r)));
-        EOD_TRY(ar.get(&h_lo, (size_t)(r4 * r)));
-        EOD_CU(split_transpose_tf32((const float *)Qb, m, r, m, q_hi, q_lo, r4, s));
-        EOD_CU(split_tf32((const float *)Rt, r, r, r, h_hi, h_lo, r4, s));
-        TcGemmDesc g;
-        g.M = m;
-        g.N = r;
-        g.K = r;
-        g.tf32 = true;
-        g.npairs = 3;
-        const TcOperand qh{q_hi, r, m, r4}, ql{q_lo, r, m, r4}, hh{h_hi, r, r, r4}, hl{h_lo, r, r, r4};
-        g.a[0] = qh, g.b[0] = hh;
-        g.a[1] = qh, g.b[1] = hl;
-        g.a[2] = ql, g.b[2] = hh;
-        g.D = (float *)U;
-        g.ldd = m;
-        g.err_flag = ws.err_flag;
-        EOD_CU(tc_gemm_run(g, &ws, s));
+    auto core_blocked = [&]() -> eod_status {
+        EOD_CU((copy_matrix<T, T>(Ct, n, V, n, n, r, false, s)));
+        EOD_TRY(cholqr2(cw, V, n, n, r, Rc, hm, &ws, s));                 // C^T = V R
+        EOD_CU((copy_matrix<double, T>(Rc, r, Qh, r, r, r, true, s)));    // R^T
+        return cholqr2(cw, Qh, r, r, r, D, hm, &ws, s);                   // R^T = Qh D
+    };
+    const bool one_leaf = core_one_leaf(r);
+    if (one_leaf) {
+        EOD_TRY(cholqr2_one_leaf(cw, Ct, V, n, r, Rc, core_info, &ws, s));
+        EOD_CU((copy_matrix<double, T>(Rc, r, Rt, r, r, r, true, s)));
+        EOD_TRY(cholqr2_one_leaf(cw, Rt, Qh, r, r, D, core_info + 4, &ws, s));
     } else {
-        EOD_CU((gemm<T, T, T, T>(false, false, m, r, r, 1.0, Qb, m, Rt, r, 0.0, U, m, ex, &ws, s)));
+        EOD_TRY(core_blocked());
     }
+    // U = Q Qh
+    auto form_u = [&]() -> eod_status {
+        if (oz.on && fp64_use_emulated(m, r, r)) {
+            const int64_t r8 = round_up8(r);
+            uint16_t *qhs;
+            int *eqh;
+            EOD_TRY(ar.get(&qhs, (size_t)kOzSlices * r * r8));
+            EOD_TRY(ar.get(&eqh, (size_t)r));
+            EOD_CU(oz_slice((const double *)Qh, r, r, r, 1, qhs, eqh, 0, r8, r * r8, s));
+            const OzOperand qr{oz.Qr, nullptr, 1, oz.cap8, m * oz.cap8};
+            const OzOperand qho{qhs, eqh, 0, r8, r * r8};
+            EOD_CU(oz_gemm_ops(qr, qho, m, r, r, 1.0, 0.0, (double *)U, m, ex, ws.err_flag, s));
+        } else if (mixed && std::is_same<T, float>::value && m >= kTfMinRows && r >= 32) {
+            // on the tensor cores as three TF32 products of split
+            // operands, X = X_hi + X_lo (X_hi Y_hi + X_hi Y_lo + X_lo Y_hi: about
+            // 2^-21 relative, the accuracy of an FP32 product); TF32 operands are
+            // K-major, so Q is split transposed (r4 x m)
+            const int64_t r4 = round_up(r, 4);
+            float *q_hi, *q_lo, *h_hi, *h_lo;
+            EOD_TRY(ar.get(&q_hi, (size_t)(r4 * m)));
+            EOD_TRY(ar.get(&q_lo, (size_t)(r4 * m)));
+            EOD_TRY(ar.get(&h_hi, (size_t)(r4 * r)));
+            EOD_TRY(ar.get(&h_lo, (size_t)(r4 * r)));
+            EOD_CU(split_transpose_tf32((const float *)Qb, m, r, m, q_hi, q_lo, r4, s));
+            EOD_CU(split_tf32((const float *)Qh, r, r, r, h_hi, h_lo, r4, s));
+            TcGemmDesc g;
+            g.M = m;
+            g.N = r;
+            g.K = r;
+            g.tf32 = true;
+            g.npairs = 3;
+            const TcOperand qh{q_hi, r, m, r4}, ql{q_lo, r, m, r4}, hh{h_hi, r, r, r4}, hl{h_lo, r, r, r4};
+            g.a[0] = qh, g.b[0] = hh;
+            g.a[1] = qh, g.b[1] = hl;
+            g.a[2] = ql, g.b[2] = hh;
+            g.D = (float *)U;
+            g.ldd = m;
+            g.err_flag = ws.err_flag;
+            EOD_CU(tc_gemm_run(g, &ws, s));
+        } else {
+            EOD_CU((gemm<T, T, T, T>(false, false, m, r, r, 1.0, Qb, m, Qh, r, 0.0, U, m, ex, &ws, s)));
+        }
+        return EOD_OK;
+    };
+    EOD_TRY(form_u());
 
+    // one host read: RelErr, the T diagonal, the core's leaves and the bounded
+    // waits' flags
     join.join();
-    if (o.compute_err) {
-        EOD_CU(cudaMemcpyAsync(hm.val, d_err, sizeof(double), cudaMemcpyDeviceToHost, s));
+    for (int round = 0;; ++round) {
+        if (o.compute_err) EOD_CU(cudaMemcpyAsync(hm.val, d_err, sizeof(double), cudaMemcpyDeviceToHost, s));
+        if (one_leaf) EOD_CU(cudaMemcpyAsync(hm.core, core_info, sizeof(int) * 8, cudaMemcpyDeviceToHost, s));
+        hm.flag[1] = 0;
+        EOD_CU(cudaMemcpyAsync(hm.flag, ws.err_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+        if (mixed) EOD_CU(mx.copy_flag(hm.flag + 1, s));
+        if (round == 0) EOD_CU(queue_tdiag());
+        EOD_CU(cudaStreamSynchronize(s));
+        if (hm.flag[0] || hm.flag[1]) return EOD_ETIMEOUT;
+        if (round == 0) EOD_TRY(finish_tdiag());
+        bool first = true, second = true;   // the leaves of the first and second passes
+        if (one_leaf && round == 0)
+            for (int q = 0; q < 2; ++q) {
+                first = first && hm.core[4 * q] == r && hm.core[4 * q + 1] == CHOL_ALL;
+                second = second && hm.core[4 * q + 2] == r && hm.core[4 * q + 3] == CHOL_ALL;
+            }
+        if (!first) {   // unshifted CholQR broke down: the blocked form takes its shifted passes
+            EOD_TRY(core_blocked());
+            EOD_TRY(form_u());
+            continue;
+        }
+        if (!second) return EOD_EPRECISION;
+        break;
     }
-    EOD_CU(cudaStreamSynchronize(s));
     F->rel_err = o.compute_err ? hm.val[0] : -1.0;
-    if (mixed) EOD_TRY(mx.check(s));
-    EOD_CU(cudaMemcpyAsync(hm.flag, ws.err_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    EOD_CU(cudaStreamSynchronize(s));
-    if (hm.flag[0]) return EOD_ETIMEOUT;
 
     F->U = U; ar.keep(U);
     F->V = V; ar.keep(V);

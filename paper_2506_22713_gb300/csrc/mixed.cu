@@ -229,12 +229,8 @@ eod_status MixedOps<float>::recon_error(const float *Q, int64_t r, const float *
     return EOD_OK;
 }
 
-eod_status MixedOps<float>::check(cudaStream_t s) {
-    if (!err_flag) return EOD_OK;
-    int h = 0;
-    MX_TRY(cudaMemcpyAsync(&h, err_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
-    MX_TRY(cudaStreamSynchronize(s));
-    return h ? EOD_ETIMEOUT : EOD_OK;
+cudaError_t MixedOps<float>::copy_flag(int *host, cudaStream_t s) {
+    return err_flag ? cudaMemcpyAsync(host, err_flag, sizeof(int), cudaMemcpyDeviceToHost, s) : cudaSuccess;
 }
 
 }  // namespace eod

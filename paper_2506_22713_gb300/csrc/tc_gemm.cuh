@@ -80,7 +80,7 @@ struct MixedOps {
     eod_status recon_error(const T *, int64_t, const T *, const double *, double *, cudaStream_t, cudaStream_t) {
         return EOD_EUNSUPPORTED;
     }
-    eod_status check(cudaStream_t) { return EOD_OK; }
+    cudaError_t copy_flag(int *, cudaStream_t) { return cudaSuccess; }
 };
 
 template <>
@@ -111,7 +111,8 @@ struct MixedOps<float> {
     // `s`), ordered after those allocations
     eod_status recon_error(const float *Q, int64_t r, const float *Ct, const double *d_norm, double *d_err,
                            cudaStream_t s, cudaStream_t run);
-    eod_status check(cudaStream_t s);   // EOD_ETIMEOUT if a bounded device wait ran out
+    // queues the copy of the flag a bounded device wait that ran out sets
+    cudaError_t copy_flag(int *host, cudaStream_t s);
 };
 
 }  // namespace eod
