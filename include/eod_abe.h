@@ -62,11 +62,14 @@ typedef enum {
                               type.  EOD_F64: products of at least 2^25
                               multiply-adds run as an exact FP64 emulation on
                               the tcgen05 tensor cores (each operand split into
-                              eight BF16 digit slices, integer-exact partial
-                              products, FP64 accumulation; normwise error about
-                              K 2^-48 |A(i,:)| |B(:,j)|), smaller ones as FP64
-                              DFMA; EOD_F32: FP32 FFMA.  Gram/Cholesky/rank
-                              test/core in FP64 */
+                              seven BF16 digit slices, integer-exact partial
+                              products and sums, one rounding; normwise error
+                              about K 2^-54 |A(i,:)| |B(:,j)|), smaller ones as
+                              FP64 DFMA; EOD_F32: FP32 FFMA, the products with
+                              no narrow side and 2^29.5 multiply-adds or more
+                              as the same emulation with four digits, rounded
+                              once to FP32.  Gram/Cholesky/rank test/core in
+                              FP64 */
     EOD_MIXED_BF16 = 1,    /* sketch, projection and reconstruction on tcgen05
                               tensor cores with FP32 accumulation: A split into
                               three BF16 terms for the sketch (exact for FP32

@@ -199,8 +199,7 @@ struct OzOperand {
     int64_t ldk = 0, slice_stride = 0;
 };
 cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha,
-                        double beta, double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s,
-                        float *Cf = nullptr);
+                        double beta, double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s);
 // FP32 data through the same emulation (FP32 values are exact in FP64), the
 // result rounded once to FP32: C = alpha op(A) op(B) + beta C (EPI_STORE only)
 cudaError_t oz_gemm_f32(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const float *A, int64_t lda,
@@ -213,6 +212,7 @@ cudaError_t oz_slice(const double *X, int64_t rows, int64_t K, int64_t sr, int64
                      int fixed_e, int64_t ldk, int64_t slice_stride, cudaStream_t s);
 constexpr int kOzSlices = 7;       // the factorisation's products
 constexpr int kOzSlicesFine = 8;   // GemmExtra::fine
+constexpr int kOzSlicesF32 = 4;    // FP32 data and result (oz_gemm_f32)
 
 // whether gemm<double,...> sends an M x N x K product to oz_gemm
 bool fp64_use_emulated(int64_t M, int64_t N, int64_t K);

@@ -1269,9 +1269,9 @@ static eod_status reconstruct_impl(const eod_factors *f, T *Ahat, int64_t ld, cu
         const cudaError_t e = gemm<T, T, T, T>(false, false, m, r, r, 1.0, U, m, Dt, r, 0.0, W, m, bu, &ws, s);   // W = U D
         return e != cudaSuccess ? e : gemm<T, T, T, T>(false, true, m, n, r, 1.0, W, m, V, n, 0.0, Ahat, ld, ex, &ws, s);
     };
-    if (std::is_same<T, double>::value && fp64_use_emulated(m, n, r)) {
-        // FP64: the larger of the two products (or both) on the tensor cores,
-        // as in the factorisation.  The emulation takes non-finite entries for
+    if (std::is_same<T, double>::value ? fp64_use_emulated(m, n, r) : fp32_use_emulated(m, n, r)) {
+        // The larger of the two products (or both) on the tensor cores.  The
+        // emulation takes non-finite entries for
         // zero, and it needs room for the operands' slices: where either
         // happens, the DFMA products below give the result instead.
         int *flags;   // [0] a wait ran out, [1] a non-finite entry was sliced

@@ -560,18 +560,22 @@ bool fp64_use_emulated(int64_t M, int64_t N, int64_t K) {
     return (double)M * (double)N * (double)K >= 33554432.0 && K >= 8 && (M >= 128 || N >= 128);
 }
 
-// FP32 products through the emulation only with EOD_FP32_GEMM=emulated: the
-// FFMA rate is 64 times the DFMA rate, and at the shapes of the method (one
-// side at most a few hundred, FP32 operands sliced on every call) the FFMA
-// kernel measured as fast or faster (8192 x 455 x 455: 259 us FFMA against
-// 255 us emulated plus 64 us of slicing; 8192 x 256 x 256: 75 against
-// 85 + 36 us), so it stays the default.
+// Large FP32 products go to the emulation with four digits (oz_gemm.cu), whose
+// result is the exact product's rounding (relative error 2.5e-8; FFMA 1e-7 to
+// 1.3e-6), where neither side is narrow: its tiles are 128 x 64 and both
+// operands are sliced on every call.  FFMA against digits with their slicing:
+// 8192 x 8192 x 473 1515 / 875 us, 3001 x 2503 x 313 306 / 140, 2049 x 326 x
+// 1537 299 / 96, 8192 x 455 x 8192 1936 / 1144, 8192 x 455 x 455 115 / 104; and
+// below the line 8192 x 256 x 256 35 / 61, 2503 x 313 x 313 44 / 61, 8192 x 96 x
+// 384 49 / 73, 2048 x 2048 x 64 21 / 76.  EOD_FP32_GEMM=emulated sends every
+// product there.
 bool fp32_use_emulated(int64_t M, int64_t N, int64_t K) {
-    static const bool on = [] {
+    static const bool all = [] {
         const char *v = std::getenv("EOD_FP32_GEMM");
         return v && std::strcmp(v, "emulated") == 0;
     }();
-    return on && M >= 1 && N >= 1 && K >= 1;
+    if (all) return M >= 1 && N >= 1 && K >= 1;
+    return M >= 256 && N >= 256 && K > 256 && (double)M * (double)N * (double)K >= 7.6e8;   // 2^29.5
 }
 
 template <typename TA, typename TB, typename TC, typename Acc>
@@ -584,8 +588,7 @@ cudaError_t gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha
         ws && ws->err_flag && K > 0 && fp64_use_emulated(M, N, K))
         return oz_gemm(ta, tb, M, N, K, alpha, (const double *)A, lda, (const double *)B, ldb, beta, (double *)C,
                        ldc, x, ws->err_flag, s);
-    // large FP32 products: the same emulation (more accurate than FP32 FFMA
-    // and far faster on this GPU), rounded once to FP32
+    // large FP32 products: the same emulation, rounded once to FP32
     if (std::is_same<TA, float>::value && std::is_same<TB, float>::value && std::is_same<TC, float>::value &&
         ws && ws->err_flag && K > 0 && x.epilogue == EPI_STORE && fp32_use_emulated(M, N, K))
         return oz_gemm_f32(ta, tb, M, N, K, alpha, (const float *)A, lda, (const float *)B, ldb, beta, (float *)C,

@@ -22,6 +22,10 @@
 // row x column scale per term.
 //   NS = 7 (28 products): the factorisation's products; 2^-56 per term, the
 //   level of an FP64 dot product.
+//   NS = 4 (10 products): FP32 data and results; 2^-31 per term, below FP32's
+//   own rounding.  Its 4 x 64 accumulator columns fit TMEM twice, so a chunk is
+//   drained while the next is multiplied; with more tiles than SMs a CTA takes
+//   several, its products running ahead of its epilogues.
 //   NS = 8 (36 products): where the result has to be as accurate as FP64 FMAs
 //   whatever the operands' spread (A_hat = U D V^T).
 //
@@ -57,10 +61,14 @@ constexpr int A_TILE = BM * BK * 2;   // 16 KB: one slice
 constexpr int B_TILE = BN * BK * 2;   // 8 KB
 constexpr int BSTAGES = 2;            // K blocks of B in flight (NS slices each)
 template <int NS> struct Cfg {
-    static constexpr int ASTAGES = NS == 7 ? 6 : 5;   // A slices in flight
+    static constexpr int ASTAGES = NS == 4 ? 4 : NS == 7 ? 6 : 5;   // A slices in flight
+    static constexpr int NBUF = NS <= 4 ? 2 : 1;                     // accumulator sets in TMEM
     static constexpr int B_SET = NS * B_TILE;
-    static constexpr int SMEM = BSTAGES * B_SET + ASTAGES * A_TILE + 1024 + 256;
-    static_assert(BSTAGES * B_SET + ASTAGES * A_TILE >= 256 * 32 * 16, "the epilogue's staging");
+    // the sums staged for the epilogue: with NS = 4 (one accumulator, products
+    // of the next tile under way) in a place of their own
+    static constexpr int STAGING = NS == 4 ? 256 * 32 * 8 : 0;
+    static constexpr int SMEM = BSTAGES * B_SET + ASTAGES * A_TILE + STAGING + 1024 + 256;
+    static_assert(NS == 4 || BSTAGES * B_SET + ASTAGES * A_TILE >= 256 * 32 * 16, "the epilogue's staging");
 };
 constexpr int kMaxSlices = kOzSlicesFine;
 constexpr uint32_t TMEM_COLS = 512;   // NS x 64 used
@@ -87,6 +95,33 @@ struct Params {
     int *err_flag;
     int upper_only;           // store only entries with row <= col
     int a_tri, b_tri;         // op(A) / op(B) upper triangular: skip their zero K blocks
+    int64_t gm, tiles;        // NS = 4: tile rows, and the tiles a CTA strides over (0: one tile per CTA)
+};
+
+// The tile and K blocks of step t of this CTA; false past its last one.
+template <bool MANY>
+struct Tile {
+    int64_t m0, n0, kb0, kb1;
+    __device__ __forceinline__ bool at(const Params &p, int64_t t) {
+        if (MANY && p.tiles > 0) {
+            const int64_t i = blockIdx.x + t * gridDim.x;
+            if (i >= p.tiles) return false;
+            n0 = i / p.gm;
+            m0 = (i - n0 * p.gm) * BM;
+            n0 *= BN;
+        } else {
+            if (t > 0) return false;
+            m0 = (int64_t)blockIdx.x * BM;
+            n0 = (int64_t)blockIdx.y * BN;
+        }
+        kb0 = (int64_t)blockIdx.z * p.kb_per_split;
+        kb1 = kb0 + p.kb_per_split;
+        if (kb1 > p.kblocks) kb1 = p.kblocks;
+        if (p.a_tri && kb0 < m0 / BK) kb0 = m0 / BK;              // op(A)(i, k) = 0 for k < i
+        if (p.b_tri && kb1 > (n0 + BN + BK - 1) / BK) kb1 = (n0 + BN + BK - 1) / BK;   // op(B)(k, j) = 0 for k > j
+        if (kb1 < kb0 || (p.upper_only && m0 >= n0 + BN)) kb1 = kb0;
+        return true;
+    }
 };
 
 // m 2^e for a result outside the normal range's middle (kept out of line: its
@@ -127,6 +162,22 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
     return sign ? -v : v;
 }
 
+// h 2^e as a float, rounded once to nearest (ties to even); |h| < 2^63
+__device__ __forceinline__ float fixed_to_float(long long h, int e) {
+    if (h == 0) return 0.f;
+    const unsigned int sign = h < 0 ? 0x80000000u : 0u;
+    const unsigned long long a = h < 0 ? (unsigned long long)-h : (unsigned long long)h;
+    const int lz = __clzll((long long)a);
+    const unsigned long long m = a << lz;
+    const int ex = 63 - lz + e;                                             // value = m 2^(ex - 63)
+    // the upper 32 bits with the rest sticky, then to 24 bits
+    const unsigned int u = (unsigned int)(m >> 32) | ((unsigned int)m ? 1u : 0u);
+    const unsigned int q = (u >> 8) + ((u & 0x80u) && (u & 0x17fu) ? 1u : 0u);   // may carry to 2^24
+    if (ex >= -126 && ex <= 126) return __uint_as_float((((unsigned int)(ex + 126) << 23) + q) | sign);
+    const float v = (float)far_scale(m, ex - 63);                           // overflow or subnormal
+    return sign ? -v : v;
+}
+
 // acc + v 2^k (exact), one wide multiply-add
 __device__ __forceinline__ long long mad_wide(int v, int pow2, long long acc) {
     long long d;
@@ -136,36 +187,32 @@ __device__ __forceinline__ long long mad_wide(int v, int pow2, long long acc) {
 
 template <int NS, int EPI>
 __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_constant__ Maps maps, Params p) {
-    constexpr int NG = NS, ASTAGES = Cfg<NS>::ASTAGES, B_SET = Cfg<NS>::B_SET;
+    constexpr int NG = NS, ASTAGES = Cfg<NS>::ASTAGES, B_SET = Cfg<NS>::B_SET, NBUF = Cfg<NS>::NBUF;
+    constexpr uint32_t BUF_COLS = TMEM_COLS / NBUF;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *bbuf = smem;                                 // BSTAGES x NS B slices
     uint8_t *abuf = smem + BSTAGES * B_SET;                // ring of A slices
-    uint64_t *fullB = (uint64_t *)(abuf + ASTAGES * A_TILE);
+    uint64_t *fullB = (uint64_t *)(abuf + ASTAGES * A_TILE + Cfg<NS>::STAGING);
     uint64_t *emptyB = fullB + BSTAGES;
     uint64_t *fullA = emptyB + BSTAGES;
     uint64_t *emptyA = fullA + ASTAGES;
     uint64_t *tmem_full = emptyA + ASTAGES;
-    uint64_t *tmem_empty = tmem_full + 1;
-    uint32_t *tmem_slot = (uint32_t *)(tmem_empty + 1);
+    uint64_t *tmem_empty = tmem_full + NBUF;
+    uint32_t *tmem_slot = (uint32_t *)(tmem_empty + NBUF);
     int *abort_sh = (int *)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t m0 = (int64_t)blockIdx.x * BM, n0 = (int64_t)blockIdx.y * BN;
-    if (p.upper_only && m0 >= n0 + BN) return;   // every entry of the tile is below the diagonal
-    int64_t kb0 = (int64_t)blockIdx.z * p.kb_per_split;
-    int64_t kb1 = kb0 + p.kb_per_split;
-    if (kb1 > p.kblocks) kb1 = p.kblocks;
-    if (p.a_tri && kb0 < m0 / BK) kb0 = m0 / BK;              // op(A)(i, k) = 0 for k < i
-    if (p.b_tri && kb1 > (n0 + BN + BK - 1) / BK) kb1 = (n0 + BN + BK - 1) / BK;   // op(B)(k, j) = 0 for k > j
-    const int64_t nkb = kb1 > kb0 ? kb1 - kb0 : 0;
-    const int64_t nchunks = (nkb + KCH - 1) / KCH;
+    Tile<NS == kOzSlicesF32> w;
+    if (!(NS == kOzSlicesF32 && p.tiles > 0) && p.upper_only) {   // every entry of the tile is below the diagonal
+        w.at(p, 0);
+        if (w.m0 >= w.n0 + BN) return;
+    }
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < BSTAGES; ++i) { mbar_init(&fullB[i], 1); mbar_init(&emptyB[i], 1); }
         for (int i = 0; i < ASTAGES; ++i) { mbar_init(&fullA[i], 1); mbar_init(&emptyA[i], 1); }
-        mbar_init(tmem_full, 1);
-        mbar_init(tmem_empty, 256);
+        for (int i = 0; i < NBUF; ++i) { mbar_init(&tmem_full[i], 1); mbar_init(&tmem_empty[i], 256); }
         *abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -187,15 +234,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         const bool leader = elect_one();
         int64_t ib = 0, ia = 0;
         bool ok = true;
-        for (int64_t kb = kb0; kb < kb1 && ok; ++kb) {
+        for (int64_t t = 0; ok && w.at(p, t); ++t)
+        for (int64_t kb = w.kb0; kb < w.kb1 && ok; ++kb) {
             const int sb = (int)(ib % BSTAGES);
             if (ib >= BSTAGES) ok = warp_wait(&emptyB[sb], (uint32_t)((ib / BSTAGES - 1) & 1));
             if (ok && __any_sync(0xffffffffu, *(volatile int *)abort_sh != 0)) ok = false;
             if (!ok) break;
             if (leader) {
                 mbar_expect_tx(&fullB[sb], B_SET);
-                for (int t = 0; t < NS; ++t)
-                    tma_load_2d(bbuf + sb * B_SET + t * B_TILE, &maps.b[t], &fullB[sb], (int)(kb * BK), (int)n0);
+                for (int q = 0; q < NS; ++q)
+                    tma_load_2d(bbuf + sb * B_SET + q * B_TILE, &maps.b[q], &fullB[sb], (int)(kb * BK), (int)w.n0);
             }
             ++ib;
             for (int s = 0; s < NS && ok; ++s) {
@@ -204,7 +252,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                 if (!ok) break;
                 if (leader) {
                     mbar_expect_tx(&fullA[sa], A_TILE);
-                    tma_load_2d(abuf + sa * A_TILE, &maps.a[s], &fullA[sa], (int)(kb * BK), (int)m0);
+                    tma_load_2d(abuf + sa * A_TILE, &maps.a[s], &fullA[sa], (int)(kb * BK), (int)w.m0);
                 }
                 ++ia;
             }
@@ -223,11 +271,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         constexpr uint32_t idesc = idesc_bf16(BM, BN, false, false);
         int64_t ib = 0, ia = 0;
         bool ok = true;
+        int64_t chunk0 = 0;   // chunks of the tiles before
+        for (int64_t step = 0; ok && w.at(p, step); ++step) {
+        const int64_t nkb = w.kb1 - w.kb0;
         for (int64_t q = 0; q < nkb && ok; ++q) {
             const bool first = (q % KCH) == 0;
+            const int64_t chunk = chunk0 + q / KCH;
+            const int buf = NBUF > 1 ? (int)(chunk % NBUF) : 0;
+            const uint32_t tacc = tmem + (uint32_t)buf * BUF_COLS;
             if (first) {
-                const int64_t chunk = q / KCH;
-                if (chunk > 0) ok = warp_wait(tmem_empty, (uint32_t)((chunk - 1) & 1));
+                if (chunk >= NBUF) ok = warp_wait(&tmem_empty[buf], (uint32_t)((chunk / NBUF - 1) & 1));
                 if (!ok) break;
                 tc_fence_after();
             }
@@ -252,7 +305,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                                 for (int kk = 0; kk < BK / UMMA_K; ++kk) {
                                     // the first MMA of a group in a chunk overwrites it
                                     const uint32_t accum = (first && s == 0 && kk == 0) ? 0u : 1u;
-                                    umma_bf16(tmem + (uint32_t)((s + t) * BN), ad0 + (uint64_t)(2 * kk),
+                                    umma_bf16(tacc + (uint32_t)((s + t) * BN), ad0 + (uint64_t)(2 * kk),
                                               bd0 + (uint64_t)(512 * t + 2 * kk), idesc, accum);
                                 }
                             }
@@ -266,20 +319,29 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
             if (!ok) break;
             if (leader) {
                 umma_commit(&emptyB[sb]);
-                if (q % KCH == KCH - 1 || q == nkb - 1) umma_commit(tmem_full);
+                if (q % KCH == KCH - 1 || q == nkb - 1) umma_commit(&tmem_full[buf]);
             }
             __syncwarp();
             ++ib;
         }
+        chunk0 += (nkb + KCH - 1) / KCH;
+        }
         if (!ok && leader) {
             atomicExch(p.err_flag, 1);
             *abort_sh = 1;
-            umma_commit(tmem_full);   // release the epilogue once the MMAs already issued finish
+            for (int i = 0; i < NBUF; ++i) umma_commit(&tmem_full[i]);   // release the epilogue once the MMAs already issued finish
         }
     } else if (warp >= 2) {
         // ---------------- drain + epilogue ----------------
         const int qtr = warp & 3;                 // TMEM lane quarter this warp may read
         const int c0 = ((warp - 2) >> 2) * ECOLS; // its half of the 64 columns
+        constexpr int SH = 8 * (NS - 4);          // from the high unit to the low one
+        constexpr int EC = 4;
+        bool ok = true;
+        double local = 0.0;
+        int64_t chunk0 = 0;                       // chunks of the tiles before
+        for (int64_t step = 0; ok && w.at(p, step); ++step) {
+        const int64_t m0 = w.m0, n0 = w.n0, nchunks = (w.kb1 - w.kb0 + KCH - 1) / KCH;
         const int64_t row = m0 + 32 * qtr + lane;
         // this lane's row exponent and the exponent of column c0 + lane, both
         // read before the products are ready
@@ -289,13 +351,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         // accumulators, groups 0-3 in base 256 (unit 2^-38 of the row x column
         // scale, |per chunk| < 2^49) and the others (unit 2^(-14 - 8 (NS - 1)),
         // < 2^50): exact, with no FP64 instruction in the drain.
-        constexpr int SH = 8 * (NS - 4);          // from the high unit to the low one
+        // (NS = 4: the first accumulator alone.)
         long long acch[ECOLS], accl[ECOLS];
 #pragma unroll
         for (int j = 0; j < ECOLS; ++j) acch[j] = accl[j] = 0;
-        bool ok = true;
-        for (int64_t c = 0; c < nchunks; ++c) {
-            ok = __all_sync(0xffffffffu, mbar_wait(tmem_full, (uint32_t)(c & 1)) ? 1 : 0) != 0;
+        for (int64_t c = chunk0; c < chunk0 + nchunks; ++c) {
+            const int buf = NBUF > 1 ? (int)(c % NBUF) : 0;
+            ok = __all_sync(0xffffffffu, mbar_wait(&tmem_full[buf], (uint32_t)((c / NBUF) & 1)) ? 1 : 0) != 0;
             if (!ok || *(volatile int *)abort_sh) { ok = false; break; }
             tc_fence_after();
             // 4 columns at a time: the 8 groups' loads are in flight together
@@ -304,7 +366,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                 uint32_t r[NG][4];
 #pragma unroll
                 for (int g = 0; g < NG; ++g)
-                    tmem_ld4_nowait(tmem + ((uint32_t)(32 * qtr) << 16) + (uint32_t)(g * BN + c0 + cc), r[g]);
+                    tmem_ld4_nowait(tmem + ((uint32_t)(32 * qtr) << 16) + (uint32_t)buf * BUF_COLS + (uint32_t)(g * BN + c0 + cc),
+                                    r[g]);
                 tmem_wait_ld();
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -317,44 +380,64 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                 }
             }
             tc_fence_before();
-            mbar_arrive(tmem_empty);
+            mbar_arrive(&tmem_empty[buf]);
         }
-        if (!ok) atomicExch(p.err_flag, 1);
-        // The sums go through shared memory (free by now: every product of this
-        // CTA has been read) so that the epilogue is a short loop; unrolled over
-        // the registers its code alone, fetched once per CTA, took 30 us.
+        chunk0 += nchunks;
+        if (!ok) {
+            atomicExch(p.err_flag, 1);
+            break;
+        }
+        // The sums go through shared memory (for NS > 4 the pipeline's, free by
+        // now: every product of this CTA has been read) so that the epilogue is
+        // a short loop; unrolled over the registers its code alone, fetched once
+        // per CTA, took 30 us.
         longlong2 *st = (longlong2 *)smem + (threadIdx.x - 64);
-        if (ok) {
+        long long *st1 = (long long *)(smem + BSTAGES * B_SET + ASTAGES * A_TILE) + (threadIdx.x - 64);
 #pragma unroll
-            for (int j = 0; j < ECOLS; ++j) st[j * 256] = make_longlong2(acch[j], accl[j]);
+        for (int j = 0; j < ECOLS; ++j) {
+            if (NS == 4) st1[j * 256] = acch[j];
+            else st[j * 256] = make_longlong2(acch[j], accl[j]);
         }
-        double local = 0.0;
         const bool split = EPI == EPI_STORE && p.split_stride > 0;
         const bool unit_alpha = p.alpha == 1.0;
         // four columns at a time: what the epilogue reads (C or the reference)
         // is loaded for all of them before the first is used
-        constexpr int EC = 4;
         const int64_t left = p.N - (n0 + c0);
 #pragma unroll 1
-        for (int cc = 0; ok && cc < ECOLS && cc < left; cc += EC) {
+        for (int cc = 0; cc < ECOLS && cc < left; cc += EC) {
             double old[EC];
+            float oldf[EC];   // NS = 4
 #pragma unroll
             for (int j = 0; j < EC; ++j) {
                 const int64_t col = n0 + c0 + cc + j;
                 const bool in = row < p.M && cc + j < left && !(p.upper_only && row > col);
+                if (NS == 4) {
+                    oldf[j] = EPI == EPI_STORE && !split && p.beta != 0.0 && in ? p.Cf[row + col * p.ldc] : 0.f;
+                    continue;
+                }
                 old[j] = 0.0;
                 if (EPI == EPI_ERR) {
                     if (in) old[j] = __ldcs(p.R + row + col * p.ldr);
                 } else if (!split && p.beta != 0.0 && in) {
-                    old[j] = p.Cf ? (double)p.Cf[row + col * p.ldc] : p.C[row + col * p.ldc];
+                    old[j] = p.C[row + col * p.ldc];
                 }
             }
 #pragma unroll
             for (int j = 0; j < EC; ++j) {
                 const int64_t col = n0 + c0 + cc + j;
                 const int ec = __shfl_sync(0xffffffffu, ecol, cc + j);
-                const longlong2 v = st[(cc + j) * 256];
-                const double val = fixed_to_double<SH>(v.x, v.y, erow + ec - 14 - 8 * (NS - 1));
+                const longlong2 v = NS == 4 ? make_longlong2(st1[(cc + j) * 256], 0) : st[(cc + j) * 256];
+                const int ev = erow + ec - 14 - 8 * (NS - 1);
+                if (NS == 4 && EPI == EPI_STORE && !split) {   // an FP32 result, in FP32
+                    if (row < p.M && cc + j < left && !(p.upper_only && row > col)) {
+                        float out = fixed_to_float(v.x, ev);
+                        if (!unit_alpha) out *= (float)p.alpha;
+                        if (p.beta != 0.0) out = fmaf((float)p.beta, oldf[j], out);
+                        p.Cf[row + col * p.ldc] = out;
+                    }
+                    continue;
+                }
+                const double val = fixed_to_double<SH>(v.x, v.y, ev);
                 if (row < p.M && cc + j < left && !(p.upper_only && row > col)) {
                     if (EPI == EPI_STORE) {
                         if (split) {
@@ -362,8 +445,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                         } else {
                             double out = unit_alpha ? val : p.alpha * val;
                             if (p.beta != 0.0) out = fma(p.beta, old[j], out);
-                            if (p.Cf) p.Cf[row + col * p.ldc] = (float)out;
-                            else p.C[row + col * p.ldc] = out;
+                            p.C[row + col * p.ldc] = out;
                         }
                     } else {
                         const double d = fma(-p.alpha, val, old[j]);
@@ -371,6 +453,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
                     }
                 }
             }
+        }
         }
         if (EPI == EPI_ERR) {
             local = warp_sum(local);
@@ -400,8 +483,20 @@ __device__ __forceinline__ bool tri_zero(int tri, int64_t r, int64_t k) {
     return (tri == 1 && r > k) || (tri == 2 && k > r);
 }
 
-// |x| as its bit pattern (orders like the value for non-negative doubles);
+// |x| as its bit pattern (orders like the value for non-negative numbers);
 // non-finite entries count as zero (the contraction expects finite data).
+// FP32 data stays on the integer units: a conversion to FP64 costs a warp as
+// much as an FP64 operation.
+__device__ __forceinline__ unsigned int abs_bits(float x) {
+    const unsigned int a = __float_as_uint(x) & 0x7fffffffu;
+    return (a >> 23) == 0xff ? 0u : a;
+}
+__device__ __forceinline__ int exp_of_bits(unsigned int a) {
+    const int E = (int)(a >> 23);
+    return E > 0 ? E - 126 : -117 - __clz(a);   // subnormal: a 2^-149 < 2^(32 - clz - 149)
+}
+template <typename TX> struct AbsKey { using type = unsigned long long; };
+template <> struct AbsKey<float> { using type = unsigned int; };
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
     const unsigned long long a = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
     return (a >> 52) == 0x7ff ? 0ull : a;
@@ -428,7 +523,8 @@ template <typename TX>
 __global__ void rowexp_kernel(const TX *__restrict__ X, int64_t R, int64_t K, int64_t sr, int64_t sk,
                               int64_t kper, int tri, int *ep) {
     int *e = ep + (int64_t)blockIdx.y * R;
-    __shared__ unsigned long long red[8][33];
+    using Key = typename AbsKey<TX>::type;
+    __shared__ Key red[8][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8
     const int64_t r0 = (int64_t)blockIdx.x * 32;
     const int64_t kb = (int64_t)blockIdx.y * kper;
@@ -438,29 +534,44 @@ __global__ void rowexp_kernel(const TX *__restrict__ X, int64_t R, int64_t K, in
         // K contiguous: lanes along k, warps over rows
         for (int rr = ty; rr < 32; rr += 8) {
             const int64_t r = r0 + rr;
-            unsigned long long m = 0ull;
+            Key m = 0;
             if (r < R)
                 for (int64_t k = kb + tx; k < ke; k += 32)
-                    if (!tri_zero(tri, r, k)) m = max(m, abs_bits((double)X[r * sr + k]));
+                    if (!tri_zero(tri, r, k)) m = max(m, abs_bits(X[r * sr + k]));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (tx == 0 && r < R) e[r] = m > 0ull ? exp_of_bits(m) : kExpZero;
+            if (tx == 0 && r < R) e[r] = m > 0 ? exp_of_bits(m) : kExpZero;
         }
         return;
     }
     // rows contiguous: lanes along rows, warps split the K range
     const int64_t r = r0 + tx;
-    unsigned long long mx = 0ull;
+    Key mx = 0;
     if (r < R)
         for (int64_t k = kb + ty; k < ke; k += 8)
-            if (!tri_zero(tri, r, k)) mx = max(mx, abs_bits((double)X[r + k * sk]));
+            if (!tri_zero(tri, r, k)) mx = max(mx, abs_bits(X[r + k * sk]));
     red[ty][tx] = mx;
     __syncthreads();
     if (ty == 0 && r < R) {
-        unsigned long long m = red[0][tx];
+        Key m = red[0][tx];
 #pragma unroll
         for (int i = 1; i < 8; ++i) m = max(m, red[i][tx]);
-        e[r] = m > 0ull ? exp_of_bits(m) : kExpZero;
+        e[r] = m > 0 ? exp_of_bits(m) : kExpZero;
+    }
+}
+
+// v (below 2^(8 NS - 1)) in NS balanced base-256 digits
+template <int NS>
+__device__ __forceinline__ void cut(unsigned long long v, bool neg, __nv_bfloat16 q[NS]) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        const int w = 8 * (NS - 1 - s);
+        int d;                           // balanced digit, |d| <= 128; carries in two's complement
+        if (s == 0) d = (int)((v + (1ull << (w - 1))) >> w);
+        else if (w > 0) d = (int)((long long)(v + (1ull << (w - 1))) >> w);
+        else d = (int)(long long)v;
+        v -= (unsigned long long)(long long)d << w;
+        q[s] = __float2bfloat16_rn((float)(neg ? -d : d));
     }
 }
 
@@ -469,7 +580,6 @@ __global__ void rowexp_kernel(const TX *__restrict__ X, int64_t R, int64_t K, in
 template <int NS>
 __device__ __forceinline__ void digits(double x, int er, __nv_bfloat16 q[NS], bool &nonfinite) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-    const bool neg = (bits >> 63) != 0;
     int E = (int)((bits >> 52) & 0x7ff);
     unsigned long long M = bits & 0xfffffffffffffull;
     if (E == 0x7ff) {                    // non-finite: not representable, taken as zero
@@ -477,22 +587,31 @@ __device__ __forceinline__ void digits(double x, int er, __nv_bfloat16 q[NS], bo
         nonfinite = true;
     } else if (E == 0) E = 1;            // subnormal: M 2^(1 - 1075)
     else M |= 1ull << 52;                // |x| = M 2^(E - 1075)
-    unsigned long long v = 0;            // below 2^(8 NS - 1); the digits' carries in two's complement
+    unsigned long long v = 0;
     const int sh = E - 1075 + 8 * NS - 1 - er;   // v = M 2^sh; sh <= 8 NS - 54 since |x| < 2^er
     if (er >= -1100 && M != 0) {
         if (sh >= 0) v = M << sh;
         else if (sh > -63) v = (M >> (-sh)) + ((M >> (-sh - 1)) & 1ull);
     }
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-        const int w = 8 * (NS - 1 - s);
-        int d;                           // balanced digit, |d| <= 128
-        if (s == 0) d = (int)((v + (1ull << (w - 1))) >> w);
-        else if (w > 0) d = (int)((long long)(v + (1ull << (w - 1))) >> w);
-        else d = (int)(long long)v;
-        v -= (unsigned long long)(long long)d << w;
-        q[s] = __float2bfloat16_rn((float)(neg ? -d : d));
+    cut<NS>(v, (bits >> 63) != 0, q);
+}
+template <int NS>
+__device__ __forceinline__ void digits(float x, int er, __nv_bfloat16 q[NS], bool &nonfinite) {
+    const unsigned int bits = __float_as_uint(x);
+    int E = (int)((bits >> 23) & 0xff);
+    unsigned int M = bits & 0x7fffffu;
+    if (E == 0xff) {
+        M = 0;
+        nonfinite = true;
+    } else if (E == 0) E = 1;            // |x| = M 2^(E - 150)
+    else M |= 1u << 23;
+    unsigned long long v = 0;
+    const int sh = E - 150 + 8 * NS - 1 - er;    // sh <= 8 NS - 25
+    if (er >= -1100 && M != 0) {
+        if (sh >= 0) v = (unsigned long long)M << sh;
+        else if (sh > -31) v = (M >> (-sh)) + ((M >> (-sh - 1)) & 1u);
     }
+    cut<NS>(v, (bits >> 31) != 0, q);
 }
 
 // out[s][r * ldk + k] = slice s of X(r, k) 2^-e[r], tiles of 32 rows x 64 k
@@ -505,7 +624,7 @@ template <typename TX, int NS>
 __global__ void __launch_bounds__(256) slice_kernel(const TX *__restrict__ X, int64_t R, int64_t K, int64_t sr, int64_t sk,
                              int tri, const int *__restrict__ ep, int nsplit, int *__restrict__ e_out, int fixed_e,
                              __nv_bfloat16 *__restrict__ out, int64_t ldk, int64_t slice_stride, int *nonfinite) {
-    __shared__ double tile[32][65];
+    __shared__ TX tile[32][65];
     __shared__ int erow[32];
     const int64_t r0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * 64;
     const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
@@ -524,14 +643,14 @@ __global__ void __launch_bounds__(256) slice_kernel(const TX *__restrict__ X, in
         for (int u = 0; u < 8; ++u) {
             const int i = ty + 8 * (u >> 1), kk = tx + 32 * (u & 1);
             const int64_t r = r0 + i, k = k0 + kk;
-            tile[i][kk] = (r < R && k < K && !tri_zero(tri, r, k)) ? (double)X[r * sr + k] : 0.0;
+            tile[i][kk] = (r < R && k < K && !tri_zero(tri, r, k)) ? X[r * sr + k] : TX(0);
         }
     } else {
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int kk = ty + 8 * u;
             const int64_t r = r0 + tx, k = k0 + kk;
-            tile[tx][kk] = (r < R && k < K && !tri_zero(tri, r, k)) ? (double)X[r * sr + k * sk] : 0.0;
+            tile[tx][kk] = (r < R && k < K && !tri_zero(tri, r, k)) ? X[r * sr + k * sk] : TX(0);
         }
     }
     __syncthreads();
@@ -569,20 +688,21 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const TX *__restrict__ 
                                                          __nv_bfloat16 *__restrict__ out, int64_t ldk,
                                                          int64_t slice_stride, int *nonfinite) {
     constexpr int RU = 4;
-    __shared__ unsigned long long red[8];
+    using Key = typename AbsKey<TX>::type;
+    __shared__ Key red[8];
     __shared__ int er_sh;
     const int64_t r = blockIdx.x;
     const TX *x = X + r * sr;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t k0 = 2 * tid;
-    auto load = [&](int64_t k) -> double { return k < K && !tri_zero(tri, r, k) ? (double)x[k] : 0.0; };
-    double va[RU], vb[RU];
+    auto load = [&](int64_t k) -> TX { return k < K && !tri_zero(tri, r, k) ? x[k] : TX(0); };
+    TX va[RU], vb[RU];
 #pragma unroll
     for (int u = 0; u < RU; ++u) {
         va[u] = load(k0 + 512 * u);
         vb[u] = load(k0 + 512 * u + 1);
     }
-    unsigned long long m = 0ull;
+    Key m = 0;
 #pragma unroll
     for (int u = 0; u < RU; ++u) m = max(m, max(abs_bits(va[u]), abs_bits(vb[u])));
     for (int64_t k = k0 + 512 * RU; k < K; k += 512) m = max(m, max(abs_bits(load(k)), abs_bits(load(k + 1))));
@@ -591,10 +711,10 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const TX *__restrict__ 
     if (lane == 0) red[warp] = m;
     __syncthreads();
     if (tid == 0) {
-        unsigned long long t = red[0];
+        Key t = red[0];
 #pragma unroll
         for (int i = 1; i < 8; ++i) t = max(t, red[i]);
-        const int er = t > 0ull ? exp_of_bits(t) : kExpZero;
+        const int er = t > 0 ? exp_of_bits(t) : kExpZero;
         er_sh = er;
         e_out[r] = er;
     }
@@ -603,7 +723,7 @@ __global__ void __launch_bounds__(256) slice_rows_kernel(const TX *__restrict__ 
     __nv_bfloat16 *row = out + r * ldk;
     const bool pairs = (((uintptr_t)row | (uintptr_t)(slice_stride * 2)) & 3) == 0;
     bool bad = false;
-    auto store = [&](int64_t k, double p, double q) {
+    auto store = [&](int64_t k, TX p, TX q) {
         __nv_bfloat16 a[NS], b[NS];
         digits<NS>(p, er, a, bad);
         digits<NS>(q, er, b, bad);
@@ -719,7 +839,7 @@ template <int NS>
 cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha, double beta,
                     double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s, float *Cf) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    if (Cf && x.epilogue != EPI_STORE) return cudaErrorInvalidValue;
+    if ((NS == kOzSlicesF32) != (Cf != nullptr) || (Cf && x.epilogue != EPI_STORE)) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
     Maps maps;
     std::memset(&maps, 0, sizeof(maps));
@@ -765,7 +885,8 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
     double *part = nullptr;
     constexpr int SMEM = Cfg<NS>::SMEM;
     e = set_smem_once(oz_gemm_kernel<NS, EPI_STORE>, SMEM);
-    if (e == cudaSuccess) e = set_smem_once(oz_gemm_kernel<NS, EPI_ERR>, SMEM);
+    if constexpr (NS != kOzSlicesF32)
+        if (e == cudaSuccess) e = set_smem_once(oz_gemm_kernel<NS, EPI_ERR>, SMEM);
     if (e == cudaSuccess && splits > 1) {
         e = lib_malloc_async((void **)&part, sizeof(double) * (size_t)splits * M * N, s);
         p.C = part;
@@ -787,9 +908,18 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
                    2.0 * NS * ((double)M * K + (double)K * N) + 8.0 * 2 * M * N, s);
     if (e == cudaSuccess) {
         dim3 grid((unsigned)((M + BM - 1) / BM), (unsigned)((N + BN - 1) / BN), (unsigned)splits);
+        p.gm = grid.x;
+        if (NS == kOzSlicesF32 && splits == 1 && tiles > kNumSMs) {
+            p.tiles = tiles;
+            grid = dim3(kNumSMs);
+        }
         count_launch();
-        if (x.epilogue == EPI_ERR) oz_gemm_kernel<NS, EPI_ERR><<<grid, NTHREADS, SMEM, s>>>(maps, p);
-        else oz_gemm_kernel<NS, EPI_STORE><<<grid, NTHREADS, SMEM, s>>>(maps, p);
+        if constexpr (NS == kOzSlicesF32) {
+            oz_gemm_kernel<NS, EPI_STORE><<<grid, NTHREADS, SMEM, s>>>(maps, p);
+        } else {
+            if (x.epilogue == EPI_ERR) oz_gemm_kernel<NS, EPI_ERR><<<grid, NTHREADS, SMEM, s>>>(maps, p);
+            else oz_gemm_kernel<NS, EPI_STORE><<<grid, NTHREADS, SMEM, s>>>(maps, p);
+        }
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && splits > 1) {
@@ -807,9 +937,8 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
 }  // namespace oz
 
 cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha,
-                        double beta, double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s,
-                        float *Cf) {
-    return oz::run_ops<kOzSlices>(A, B, M, N, K, alpha, beta, C, ldc, x, err_flag, s, Cf);
+                        double beta, double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s) {
+    return oz::run_ops<kOzSlices>(A, B, M, N, K, alpha, beta, C, ldc, x, err_flag, s, nullptr);
 }
 
 namespace oz {
@@ -854,7 +983,7 @@ cudaError_t oz_gemm_f32(bool ta, bool tb, int64_t M, int64_t N, int64_t K, doubl
                         const float *B, int64_t ldb, double beta, float *C, int64_t ldc, const GemmExtra &x,
                         int *err_flag, cudaStream_t s) {
     if (x.epilogue != EPI_STORE) return cudaErrorInvalidValue;
-    return oz::gemm_any<kOzSlices, float>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, nullptr, C, ldc, x, err_flag, s);
+    return oz::gemm_any<kOzSlicesF32, float>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, nullptr, C, ldc, x, err_flag, s);
 }
 
 int64_t oz_gemm_err_ctas(int64_t M, int64_t N) { return ((M + oz::BM - 1) / oz::BM) * ((N + oz::BN - 1) / oz::BN); }

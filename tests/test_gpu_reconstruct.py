@@ -1,5 +1,6 @@
 """A_hat = U D V^T (eod_abe_reconstruct) on factor sets that a program fills
-itself, FP64 below and above the size from which its products run on the
+itself: FP32 integers, whose product has to be rounded once where it runs on
+the tensor cores (narrowest side 256, K above 256, 2^29.5 multiply-adds), and FP64 below and above the size from which its products run on the
 tensor cores (2^25 multiply-adds): odd sizes, a padded leading dimension, rank
 1, and factors that hold NaN and infinities (those propagate as with FP64
 FMAs).
@@ -36,10 +37,11 @@ def _factors(m, n, r, seed):
 
 def _run(eod, U, D, V, ld):
     m, n, r = U.shape[0], V.shape[0], D.shape[0]
-    f = eod.EodFactors(m=m, n=n, rank=r, precision=eod.EOD_PLAIN, f_dtype=eod.EOD_F64)
+    dt = eod.EOD_F64 if U.dtype == torch.float64 else eod.EOD_F32
+    f = eod.EodFactors(m=m, n=n, rank=r, precision=eod.EOD_PLAIN, f_dtype=dt)
     f.U, f.D, f.V = U.data_ptr(), D.data_ptr(), V.data_ptr()
-    out = torch.full((n, ld), -7.0, dtype=torch.float64, device="cuda")
-    o = eod.make_opts(dtype=eod.EOD_F64)
+    out = torch.full((n, ld), -7.0, dtype=U.dtype, device="cuda")
+    o = eod.make_opts(dtype=dt)
     assert eod.eod_abe_reconstruct(ctypes.byref(f), ctypes.c_void_p(out.data_ptr()), ld, ctypes.byref(o)) == eod.EOD_OK
     torch.cuda.synchronize()
     assert torch.all(out[:, m:] == -7.0)      # the padding is not written
@@ -57,15 +59,32 @@ def test_reconstruct_f64(eod, m, n, r, pad):
     assert bool(((got - ref).abs() <= bound).all())
 
 
+@pytest.mark.parametrize("m,n,r,pad", [(300, 8500, 300, 1), (1281, 1153, 515, 0), (257, 11600, 257, 3),
+                                       (5003, 300, 511, 0)])
+def test_reconstruct_f32_integers_are_rounded_once(eod, m, n, r, pad):
+    """U, V of integers below 2^12, D a diagonal of powers of two: the exact
+    sums (below 2^40) rounded to FP32."""
+    rng = np.random.default_rng(m)
+    U, V = (rng.integers(-4095, 4096, (k, r)) for k in (m, n))
+    d = 2 ** rng.integers(0, 6, r)
+    col = lambda X: torch.from_numpy(np.asfortranarray(X)).cuda()
+    got = _run(eod, col(U.astype(np.float32)), col(np.diag(d.astype(np.float64))), col(V.astype(np.float32)), m + pad)
+    ref = ((U * d).astype(np.float64) @ V.T.astype(np.float64)).astype(np.float32)
+    assert np.array_equal(got.cpu().numpy(), ref)
+
+
 @pytest.mark.parametrize("where", ["U", "D", "V"])
-def test_non_finite_factors_propagate(eod, where):
-    m, n, r = 700, 600, 150
+@pytest.mark.parametrize("m,n,r,dtype", [(700, 600, 150, torch.float64), (1400, 1300, 500, torch.float32)])
+def test_non_finite_factors_propagate(eod, where, m, n, r, dtype):
     U, D, V = _factors(m, n, r, 5)
+    U, V = (X.to(dtype).t().contiguous().t() for X in (U, V))
     {"U": U, "D": D, "V": V}[where][3, 4] = float("nan") if where != "V" else float("inf")
     got = _run(eod, U, D, V, m)
-    ref = (U @ D) @ V.t()
+    ref = (U @ D.to(dtype)) @ V.t()
     assert bool(torch.equal(torch.isnan(got), torch.isnan(ref)))
     assert bool(torch.equal(torch.isinf(got), torch.isinf(ref)))
     ok = torch.isfinite(ref)
     assert not bool(ok.all())
-    assert bool(torch.allclose(got[ok], ref[ok], rtol=1e-10, atol=1e-8))
+    size = (U.abs().double() @ D.abs() @ V.abs().double().t())[ok]
+    u = U64 if dtype == torch.float64 else 2.0 ** -24
+    assert bool(((got[ok].double() - ref[ok].double()).abs() <= 4 * (r + 2) * u * size).all())
