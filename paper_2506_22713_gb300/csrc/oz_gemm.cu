@@ -30,17 +30,25 @@
 //   whatever the operands' spread (A_hat = U D V^T).
 //
 // CTA tile 128 x 64; a K block of 64 stages all NS B slices and streams the
-// NS A slices through a ring; TMEM holds NS x 64 FP32 group accumulators.
-// Warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: drain and epilogue
-// (two per TMEM lane quarter, 32 columns each).  All waits are bounded
+// NS A slices through a ring; TMEM holds NS x 64 FP32 group accumulators.  An
+// A slice s meets all its B slices t in MMAs of up to 256 columns: the B slices
+// lie one after another in shared memory and the groups s + t in TMEM, so the A
+// rows are read once for up to four slices.  For NS > 4 the products of groups
+// 0-3 come first in every K block, then the others, and the two halves of TMEM
+// are handed over apart: the lower is drained while the chunk's last upper
+// products run, the upper while the next chunk's first lower ones do.
+// Warp 0: TMA producer, warp 1: MMA issuer, warps 2-17: drain and epilogue
+// (four per TMEM lane quarter, 16 columns each).  All waits are bounded
 // (EOD_ETIMEOUT on expiry).
 //
-// Measured (per launch, launch included): 2048^3 620 us = 27.7 TFLOP/s of FP64
-// (680 us with eight base-128 digits, 36 products and one 2^-50 accumulator),
-// 4000 x 1600 x 1600 762 us (822), slicing a 2048^2 operand and its transpose
-// 57 us (132, 2-byte stores).  What bounds it: shared-memory reads, 6 KB per
-// MMA of 128 x 64 x 16 (72 cycles each instead of 32), then the drain, about
-// 7000 cycles per chunk of integer conversions and wide additions.
+// Measured (the kernel alone): 2048^3 373 us = 46 TFLOP/s of FP64, 4000 x 1600
+// x 1600 459 us, 4000 x 1600 x 4000 999 us.  With one MMA of 64 columns per
+// slice pair (72 cycles each instead of 32: shared-memory reads, 6 KB per MMA),
+// eight drain warps and one hand-over per chunk: 634, 776 and 1750 us; wide MMAs
+// alone 452, 563 and 1209; with sixteen drain warps 429, 530 and 1173.  What
+// bounds it now: shared-memory reads (4.4 thousand cycles of a K block's about
+// 5, the MMAs alone 3.6), the first and last chunk's drain, and the last wave
+// of tiles.  Slicing a 2048^2 operand and its transpose: 57 us.
 #include "common.cuh"
 #include "instrument.cuh"
 #include "tc_gemm.cuh"
@@ -61,8 +69,9 @@ constexpr int A_TILE = BM * BK * 2;   // 16 KB: one slice
 constexpr int B_TILE = BN * BK * 2;   // 8 KB
 constexpr int BSTAGES = 2;            // K blocks of B in flight (NS slices each)
 template <int NS> struct Cfg {
-    static constexpr int ASTAGES = NS == 4 ? 4 : NS == 7 ? 6 : 5;   // A slices in flight
+    static constexpr int ASTAGES = NS == 4 ? 4 : NS == 7 ? 7 : 5;   // A slices in flight (at least 5 for NS > 4)
     static constexpr int NBUF = NS <= 4 ? 2 : 1;                     // accumulator sets in TMEM
+    static constexpr int HALVES = NS <= 4 ? 1 : 2;                   // groups 0-3 and the rest, handed over apart
     static constexpr int B_SET = NS * B_TILE;
     // the sums staged for the epilogue: with NS = 4 (one accumulator, products
     // of the next tile under way) in a place of their own
@@ -72,8 +81,9 @@ template <int NS> struct Cfg {
 };
 constexpr int kMaxSlices = kOzSlicesFine;
 constexpr uint32_t TMEM_COLS = 512;   // NS x 64 used
-constexpr int NTHREADS = 320;        // producer, MMA issuer, 8 drain warps
-constexpr int ECOLS = BN / 2;         // columns per drain warp
+constexpr int DRAIN = 16 * 32;            // drain threads
+constexpr int NTHREADS = 64 + DRAIN;      // producer, MMA issuer, drain warps
+constexpr int ECOLS = BN * 128 / DRAIN;   // columns per drain warp
 
 struct Maps {
     CUtensorMap a[kMaxSlices];
@@ -188,6 +198,7 @@ __device__ __forceinline__ long long mad_wide(int v, int pow2, long long acc) {
 template <int NS, int EPI>
 __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_constant__ Maps maps, Params p) {
     constexpr int NG = NS, ASTAGES = Cfg<NS>::ASTAGES, B_SET = Cfg<NS>::B_SET, NBUF = Cfg<NS>::NBUF;
+    constexpr int HALVES = Cfg<NS>::HALVES, NACC = NBUF * HALVES;
     constexpr uint32_t BUF_COLS = TMEM_COLS / NBUF;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -198,8 +209,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
     uint64_t *fullA = emptyB + BSTAGES;
     uint64_t *emptyA = fullA + ASTAGES;
     uint64_t *tmem_full = emptyA + ASTAGES;
-    uint64_t *tmem_empty = tmem_full + NBUF;
-    uint32_t *tmem_slot = (uint32_t *)(tmem_empty + NBUF);
+    uint64_t *tmem_empty = tmem_full + NACC;
+    uint32_t *tmem_slot = (uint32_t *)(tmem_empty + NACC);
     int *abort_sh = (int *)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -212,7 +223,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
     if (threadIdx.x == 0) {
         for (int i = 0; i < BSTAGES; ++i) { mbar_init(&fullB[i], 1); mbar_init(&emptyB[i], 1); }
         for (int i = 0; i < ASTAGES; ++i) { mbar_init(&fullA[i], 1); mbar_init(&emptyA[i], 1); }
-        for (int i = 0; i < NBUF; ++i) { mbar_init(&tmem_full[i], 1); mbar_init(&tmem_empty[i], 256); }
+        for (int i = 0; i < NACC; ++i) { mbar_init(&tmem_full[i], 1); mbar_init(&tmem_empty[i], DRAIN); }
         *abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -268,60 +279,58 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         // unit field advances by 2 per 32-byte K step and by 512 per 8 KB B
         // slice).
         const bool leader = elect_one();
-        constexpr uint32_t idesc = idesc_bf16(BM, BN, false, false);
         int64_t ib = 0, ia = 0;
         bool ok = true;
         int64_t chunk0 = 0;   // chunks of the tiles before
         for (int64_t step = 0; ok && w.at(p, step); ++step) {
         const int64_t nkb = w.kb1 - w.kb0;
         for (int64_t q = 0; q < nkb && ok; ++q) {
-            const bool first = (q % KCH) == 0;
+            const bool first = (q % KCH) == 0, last = q % KCH == KCH - 1 || q == nkb - 1;
             const int64_t chunk = chunk0 + q / KCH;
             const int buf = NBUF > 1 ? (int)(chunk % NBUF) : 0;
             const uint32_t tacc = tmem + (uint32_t)buf * BUF_COLS;
-            if (first) {
-                if (chunk >= NBUF) ok = warp_wait(&tmem_empty[buf], (uint32_t)((chunk / NBUF - 1) & 1));
-                if (!ok) break;
-                tc_fence_after();
-            }
             const int sb = (int)(ib % BSTAGES);
             ok = warp_wait(&fullB[sb], (uint32_t)((ib / BSTAGES) & 1));
             if (!ok) break;
-            tc_fence_after();
             const uint64_t bd0 = sdesc(smem_u32(bbuf + sb * B_SET), 16, 1024);
             if (__any_sync(0xffffffffu, *(volatile int *)abort_sh != 0)) ok = false;
 #pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                const int sa = (int)(ia % ASTAGES);
-                if (ok) ok = warp_wait(&fullA[sa], (uint32_t)((ia / ASTAGES) & 1));
-                if (ok) {
-                    tc_fence_after();
-                    if (leader) {
-                        const uint64_t ad0 = sdesc(smem_u32(abuf + sa * A_TILE), 16, 1024);
+            for (int h = 0; h < HALVES; ++h) {
+                // the accumulators of this half, once the chunk before has been drained
+                if (first && ok && chunk >= NBUF)
+                    ok = warp_wait(&tmem_empty[buf + h], (uint32_t)((chunk / NBUF - 1) & 1));
+                if (ok) tc_fence_after();
+                const int s1 = h == 0 ? 4 : NS;
 #pragma unroll
-                        for (int t = 0; t < NG; ++t) {
-                            if (s + t < NG) {
+                for (int s = 0; s < s1; ++s) {
+                    const int64_t at = ia + s;
+                    const int sa = (int)(at % ASTAGES);
+                    if (ok && (h == 0 || s >= 4)) ok = warp_wait(&fullA[sa], (uint32_t)((at / ASTAGES) & 1));
+                    if (ok) {
+                        tc_fence_after();
+                        if (leader) {
+                            const uint64_t ad0 = sdesc(smem_u32(abuf + sa * A_TILE), 16, 1024);
+                            // groups g0 .. g0 + n - 1: one MMA over the n B slices that belong to them
+                            const int t0 = h == 0 || s >= 4 ? 0 : 4 - s, n = (h == 0 ? 4 : NG) - s - t0;
 #pragma unroll
-                                for (int kk = 0; kk < BK / UMMA_K; ++kk) {
-                                    // the first MMA of a group in a chunk overwrites it
-                                    const uint32_t accum = (first && s == 0 && kk == 0) ? 0u : 1u;
-                                    umma_bf16(tacc + (uint32_t)((s + t) * BN), ad0 + (uint64_t)(2 * kk),
-                                              bd0 + (uint64_t)(512 * t + 2 * kk), idesc, accum);
-                                }
+                            for (int kk = 0; kk < BK / UMMA_K; ++kk) {
+                                // the first MMA of a group in a chunk overwrites it
+                                const uint32_t accum = (first && s == 0 && kk == 0) ? 0u : 1u;
+                                umma_bf16(tacc + (uint32_t)((s + t0) * BN), ad0 + (uint64_t)(2 * kk),
+                                          bd0 + (uint64_t)(512 * t0 + 2 * kk), idesc_bf16(BM, BN * n, false, false), accum);
                             }
+                            if (h == HALVES - 1) umma_commit(&emptyA[sa]);
                         }
-                        umma_commit(&emptyA[sa]);
+                        __syncwarp();
                     }
-                    __syncwarp();
                 }
-                ++ia;
+                if (!ok) break;
+                if (leader && last) umma_commit(&tmem_full[buf + h]);
             }
             if (!ok) break;
-            if (leader) {
-                umma_commit(&emptyB[sb]);
-                if (q % KCH == KCH - 1 || q == nkb - 1) umma_commit(&tmem_full[buf]);
-            }
+            if (leader) umma_commit(&emptyB[sb]);
             __syncwarp();
+            ia += NS;
             ++ib;
         }
         chunk0 += (nkb + KCH - 1) / KCH;
@@ -329,12 +338,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         if (!ok && leader) {
             atomicExch(p.err_flag, 1);
             *abort_sh = 1;
-            for (int i = 0; i < NBUF; ++i) umma_commit(&tmem_full[i]);   // release the epilogue once the MMAs already issued finish
+            for (int i = 0; i < NACC; ++i) umma_commit(&tmem_full[i]);   // release the epilogue once the MMAs already issued finish
         }
     } else if (warp >= 2) {
         // ---------------- drain + epilogue ----------------
         const int qtr = warp & 3;                 // TMEM lane quarter this warp may read
-        const int c0 = ((warp - 2) >> 2) * ECOLS; // its half of the 64 columns
+        const int c0 = ((warp - 2) >> 2) * ECOLS; // its columns of the 64
         constexpr int SH = 8 * (NS - 4);          // from the high unit to the low one
         constexpr int EC = 4;
         bool ok = true;
@@ -357,30 +366,37 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         for (int j = 0; j < ECOLS; ++j) acch[j] = accl[j] = 0;
         for (int64_t c = chunk0; c < chunk0 + nchunks; ++c) {
             const int buf = NBUF > 1 ? (int)(c % NBUF) : 0;
-            ok = __all_sync(0xffffffffu, mbar_wait(&tmem_full[buf], (uint32_t)((c / NBUF) & 1)) ? 1 : 0) != 0;
-            if (!ok || *(volatile int *)abort_sh) { ok = false; break; }
-            tc_fence_after();
-            // 4 columns at a time: the 8 groups' loads are in flight together
 #pragma unroll
-            for (int cc = 0; cc < ECOLS; cc += 4) {
-                uint32_t r[NG][4];
+            for (int h = 0; h < HALVES; ++h) {
+                constexpr int H0 = 4;
+                ok = __all_sync(0xffffffffu, mbar_wait(&tmem_full[buf + h], (uint32_t)((c / NBUF) & 1)) ? 1 : 0) != 0;
+                if (!ok || *(volatile int *)abort_sh) { ok = false; break; }
+                tc_fence_after();
+                const int g0 = h == 0 ? 0 : H0, ng = h == 0 ? H0 : NG - H0;
+                // 4 columns at a time: the groups' loads are in flight together
 #pragma unroll
-                for (int g = 0; g < NG; ++g)
-                    tmem_ld4_nowait(tmem + ((uint32_t)(32 * qtr) << 16) + (uint32_t)buf * BUF_COLS + (uint32_t)(g * BN + c0 + cc),
-                                    r[g]);
-                tmem_wait_ld();
+                for (int cc = 0; cc < ECOLS; cc += 4) {
+                    uint32_t r[4][4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
+                    for (int g = 0; g < ng; ++g)
+                        tmem_ld4_nowait(tmem + ((uint32_t)(32 * qtr) << 16) + (uint32_t)buf * BUF_COLS +
+                                            (uint32_t)((g0 + g) * BN + c0 + cc),
+                                        r[g]);
+                    tmem_wait_ld();
 #pragma unroll
-                    for (int g = 0; g < NG; ++g) {
-                        const int iv = __float2int_rn(__uint_as_float(r[g][j]));
-                        if (g < 4) acch[cc + j] = mad_wide(iv, 1 << (8 * (3 - g)), acch[cc + j]);
-                        else accl[cc + j] = mad_wide(iv, 1 << (8 * (NG - 1 - g)), accl[cc + j]);
+                    for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                        for (int g = 0; g < ng; ++g) {
+                            const int iv = __float2int_rn(__uint_as_float(r[g][j]));
+                            if (h == 0) acch[cc + j] = mad_wide(iv, 1 << (8 * (3 - g)), acch[cc + j]);
+                            else accl[cc + j] = mad_wide(iv, 1 << (8 * (NG - 1 - H0 - g)), accl[cc + j]);
+                        }
                     }
                 }
+                tc_fence_before();
+                mbar_arrive(&tmem_empty[buf + h]);
             }
-            tc_fence_before();
-            mbar_arrive(&tmem_empty[buf]);
+            if (!ok) break;
         }
         chunk0 += nchunks;
         if (!ok) {
@@ -395,8 +411,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         long long *st1 = (long long *)(smem + BSTAGES * B_SET + ASTAGES * A_TILE) + (threadIdx.x - 64);
 #pragma unroll
         for (int j = 0; j < ECOLS; ++j) {
-            if (NS == 4) st1[j * 256] = acch[j];
-            else st[j * 256] = make_longlong2(acch[j], accl[j]);
+            if (NS == 4) st1[j * DRAIN] = acch[j];
+            else st[j * DRAIN] = make_longlong2(acch[j], accl[j]);
         }
         const bool split = EPI == EPI_STORE && p.split_stride > 0;
         const bool unit_alpha = p.alpha == 1.0;
@@ -426,7 +442,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
             for (int j = 0; j < EC; ++j) {
                 const int64_t col = n0 + c0 + cc + j;
                 const int ec = __shfl_sync(0xffffffffu, ecol, cc + j);
-                const longlong2 v = NS == 4 ? make_longlong2(st1[(cc + j) * 256], 0) : st[(cc + j) * 256];
+                const longlong2 v = NS == 4 ? make_longlong2(st1[(cc + j) * DRAIN], 0) : st[(cc + j) * DRAIN];
                 const int ev = erow + ec - 14 - 8 * (NS - 1);
                 if (NS == 4 && EPI == EPI_STORE && !split) {   // an FP32 result, in FP32
                     if (row < p.M && cc + j < left && !(p.upper_only && row > col)) {
@@ -457,12 +473,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         }
         if (EPI == EPI_ERR) {
             local = warp_sum(local);
-            __shared__ double red[8];
+            __shared__ double red[DRAIN / 32];
             if (lane == 0) red[warp - 2] = local;
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(DRAIN) : "memory");
             if (warp == 2 && lane == 0) {
                 double t = 0.0;
-                for (int i = 0; i < 8; ++i) t += red[i];
+                for (int i = 0; i < DRAIN / 32; ++i) t += red[i];
                 p.errp[blockIdx.x + (int64_t)blockIdx.y * gridDim.x] = t;
             }
         }
