@@ -22,6 +22,12 @@
 //     next diagonal block are pushed to every CTA through distributed shared
 //     memory, one cluster barrier (about 480 cycles) each; what the next
 //     block does not need at once runs beside its factorisation.
+//   - Inside a block the entries are dealt to the lanes one by one, whatever
+//     their row: with a row to a warp most lanes idled, and the FP64 issue
+//     slots of the idle ones held up the 8-column chain (5400 cycles alone,
+//     7800 beside them, and as long again waiting for them).  A leaf of 64, 96,
+//     128 columns: 57, 86, 126 us before, 42, 68, 103 now.  Half of what is left
+//     is the 8-column chain.
 // Every CTA takes every decision on identical bits, so the barriers match.
 #pragma once
 
@@ -33,10 +39,11 @@ namespace {
 constexpr int kLB = 32;            // columns per block
 constexpr int kLBS = kLB + 1;      // odd row stride of the 32-wide buffers
 constexpr int kLeafCluster = 8;    // CTAs when the leaf is spread (portable cluster size)
-// Widths up to this run on one CTA column by column (chol_leaf.cuh): at 64
-// both take 58 us (launch included); at 80, 96, 112, 128 the cluster takes
-// 75, 90, 111, 131 us against 88, 129, 182, 250.
-constexpr int kLeafOneCta = 64;
+// Widths up to this run on one CTA column by column (chol_leaf.cuh).  Launch
+// and read back, one CTA against cluster, us: 8 26 / 27, 16 30 / 30, 20 33 / 32,
+// 24 35 / 34, 32 40 / 38, 64 76 / 59, 96 148 / 85, 128 274 / 120 (of these 16 are
+// the measurement's own).
+constexpr int kLeafOneCta = 16;
 
 __device__ __forceinline__ uint32_t leaf_smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // v into the same shared-memory place of the cluster's CTA `rank`
@@ -278,7 +285,10 @@ __global__ void __launch_bounds__(kLeafThreads) chol_block_kernel(const LeafArgs
             if (B0 == 0) return;
             const int nch = (w - B0 + 31) / 32, orow = (B1 - q + C - 1) / C;   // own rows >= B1
             const int nrow = nown > orow ? nown - orow : 0, T = (nrow + of0) * nch;
-            for (int t = T * part0 / parts + me; t < T * part1 / parts; t += nme) {
+            // one task per warp at least in the first part, where the warps have nothing else
+            const int least = T < NWK ? T : NWK;
+            const int t0 = part0 == 0 ? 0 : max(T * part0 / parts, least), t1 = max(T * part1 / parts, least);
+            for (int t = t0 + me; t < t1; t += nme) {
                 const int ch = t / (nrow + of0), oo = t - ch * (nrow + of0);
                 if (oo < nrow) {
                     const int o = nown - 1 - oo, r = q + C * o, c = B0 + 32 * ch + lane;
@@ -298,24 +308,32 @@ __global__ void __launch_bounds__(kLeafThreads) chol_block_kernel(const LeafArgs
                                      &code_sh);
                 if (lane == 0) pl_sh = pl;
             } else if (worker) {
-                left(s ? s + 1 : 0, s + 2, 5, wid, NWK);
                 if (s > 0) {
-                    // the rest of step s - 1 (columns e0 .. e0 + 7)
-                    const int e0 = c0 - 8;
-                    for (int r = c0 + 8 + wid; r < nv; r += NWK) {
-                        const int c = c0 + lane;
+                    // the rest of step s - 1 (columns e0 .. e0 + 7): entries dealt
+                    // to the lanes one by one (a row to a warp left most idle, and
+                    // an FP64 instruction costs the same for any number of lanes)
+                    const int e0 = c0 - 8, nr = nv - c0, me = wid * 32 + lane;
+                    const int inv_nr = (65535 + nr) / nr, inv_c0 = (65535 + c0) / c0;   // t / x = t inv_x >> 16 for t < 2^10
+                    for (int t = me; t < (nr - 8) * nr; t += NWK * 32) {
+                        const int k = (t * inv_nr) >> 16, r = c0 + 8 + k, c = c0 + t - k * nr;
                         if (c <= r) Sd[r * kLBS + c] -= dot8(Li + r * 9, Xi + c * 9, 1);
                     }
-                    for (int k = wid; k < 8; k += NWK)
-                        if (lane < e0) Zt[k * kLBS + lane] = dot8(Zd + (e0 + k) * kLBS + e0, Zd + e0 * kLBS + lane, kLBS);
-                    asm volatile("bar.sync 1, 384;" ::: "memory");
-                    for (int r = c0 + wid; r < nv; r += NWK) {
-                        if (lane < e0) Zd[r * kLBS + lane] -= dot8(Li + r * 9, Zt + lane, kLBS);
-                        else if (lane < c0) Zd[r * kLBS + lane] = -dot8(Li + r * 9, Zd + e0 * kLBS + lane, kLBS);
+                    if (me < 8 * e0) {              // e0 = 8 or 16
+                        const int k = me >> (e0 == 16 ? 4 : 3), c = me & (e0 - 1);
+                        Zt[k * kLBS + c] = dot8(Zd + (e0 + k) * kLBS + e0, Zd + e0 * kLBS + c, kLBS);
                     }
-                    for (int k = wid; k < 8; k += NWK)
-                        if (lane < e0) Zd[(e0 + k) * kLBS + lane] = Zt[k * kLBS + lane];
+                    asm volatile("bar.sync 1, 384;" ::: "memory");
+                    for (int t = me; t < nr * c0; t += NWK * 32) {
+                        const int k = (t * inv_c0) >> 16, r = c0 + k, c = t - k * c0;
+                        const double v = dot8(Li + r * 9, c < e0 ? Zt + c : Zd + e0 * kLBS + c, kLBS);
+                        Zd[r * kLBS + c] = (c < e0 ? Zd[r * kLBS + c] : 0.0) - v;
+                    }
+                    if (me < 8 * e0) {
+                        const int k = me >> (e0 == 16 ? 4 : 3), c = me & (e0 - 1);
+                        Zd[(e0 + k) * kLBS + c] = Zt[k * kLBS + c];
+                    }
                 }
+                left(s ? s + 1 : 0, s + 2, 5, wid, NWK);
             }
             __syncthreads();
             const int pl = pl_sh;
@@ -331,17 +349,12 @@ __global__ void __launch_bounds__(kLeafThreads) chol_block_kernel(const LeafArgs
                 __syncthreads();
                 break;
             }
-            // the 8 columns of the rows below in this block (column k on warp
-            // k or 11 - k: every sub-partition takes nine terms)
-            if (warp < 8) {
-                const int k = warp < 4 ? warp : 11 - warp, r = c0 + 8 + lane;
+            // the 8 columns of the rows below in this block (Zd is zero above its
+            // diagonal)
+            {
+                const int k = tid & 7, r = c0 + 8 + (tid >> 3);
                 if (r < nv) {
-                    const double *xs = Sd + r * kLBS + c0, *zs = Zd + (c0 + k) * kLBS + c0;
-                    double s0 = xs[0] * zs[0], s1 = 0.0;
-#pragma unroll
-                    for (int l = 1; l < 8; ++l)
-                        if (l <= k) (l & 1 ? s1 : s0) = fma(xs[l], zs[l], l & 1 ? s1 : s0);
-                    const double x = s0 + s1;
+                    const double x = dot8(Sd + r * kLBS + c0, Zd + (c0 + k) * kLBS + c0, 1);
                     Xi[r * 9 + k] = x;
                     Li[r * 9 + k] = x * di[B0 + c0 + k];
                 }

@@ -89,3 +89,25 @@ def test_block_leaf_not_positive_and_shift(eod):
     G[77, 77] = -1.0
     p, code, _, _ = _run(eod, G)
     assert code == 3 and p <= 77
+
+
+@pytest.mark.parametrize("w", [17, 24, 25, 31, 32, 33, 39, 40, 41, 57, 63, 64])
+@pytest.mark.parametrize("cond,pad", [(1e2, 0), (1e8, 3)])
+def test_block_leaf_of_one_and_two_blocks(eod, w, cond, pad):
+    """Widths of one or two blocks, whole and ragged, with the same bounds."""
+    test_block_leaf(eod, w, cond, pad)
+
+
+@pytest.mark.parametrize("w,stop", [(24, 0), (24, 8), (32, 15), (32, 31), (40, 33), (64, 20), (64, 32), (64, 63)])
+def test_narrow_block_leaf_stops_at_the_same_column(eod, w, stop):
+    rng = np.random.default_rng(100 * w + stop)
+    X = rng.standard_normal((300, w))
+    X[:, stop] = (X[:, :stop] @ rng.standard_normal(stop) if stop else 0.0) + 1e-7 * rng.standard_normal(300)
+    G = X.T @ X
+    coef = 64.0 * (w + np.sqrt(300.0)) * U64
+    for decide in (1, 257):
+        p, code, R, Ri = _run(eod, G, decide=decide, eps2=1e-6, coef=coef, rho=1e-10)
+        assert p == stop and code in (1, 2)
+        if stop:
+            assert np.linalg.norm(R.T @ R - G[:p, :p]) <= 20 * p * U64 * np.linalg.norm(G)
+            assert np.linalg.norm(Ri @ R - np.eye(p)) <= 1e-9
