@@ -623,7 +623,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     if (mixed && !norm_in_split) EOD_TRY(mx.prepare(A, m, n, lda, k, ar, &ws, s, o.precision == EOD_MIXED_TF32));
 
     OzCache oz;
-    oz.on = std::is_same<T, double>::value && fp64_use_emulated(m, k, n);
+    oz.on = std::is_same<T, double>::value && fp64_keep_slices(m, k, n);
     if (oz.on) {
         oz.m = m;
         oz.m8 = round_up8(m);
@@ -686,7 +686,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
         if (nq <= 0) return cudaSuccess;
         const T *Qq = Qb + q0 * m;
         cudaError_t e;
-        if (oz.on && fp64_use_emulated(nq, wdt, m)) {
+        if (oz.on && fp64_use_emulated_sliced(nq, wdt, m)) {
             OzOperand bo;
             e = oz_small_to(Yc, wdt, m, m, 1, bt, ebt, st, bo);
             if (e != cudaSuccess) return e;
@@ -696,7 +696,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             e = gemm<T, T, T, T>(true, false, nq, wdt, m, 1.0, Qq, m, Yc, m, 0.0, Sb, cap, ex, w, st);
         }
         if (e != cudaSuccess) return e;
-        if (oz.on && fp64_use_emulated(m, wdt, nq) && q0 % 8 == 0) {
+        if (oz.on && fp64_use_emulated_sliced(m, wdt, nq) && q0 % 8 == 0) {
             OzOperand bo;
             e = oz_small_to(Sb, wdt, nq, cap, 1, bt, ebt, st, bo);
             if (e != cudaSuccess) return e;
@@ -1018,7 +1018,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             const int64_t nct = gemm_err_ctas(m, n);
             double *part;
             EOD_TRY(ar.get(&part, (size_t)nct));
-            const bool emulated = oz.on && fp64_use_emulated(m, n, r);
+            const bool emulated = oz.on && fp64_use_emulated_sliced(m, n, r);
             uint16_t *cts = nullptr;
             int *ects = nullptr;
             const int64_t r8 = round_up8(r);
@@ -1068,7 +1068,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     }
     // U = Q Qh
     auto form_u = [&]() -> eod_status {
-        if (oz.on && fp64_use_emulated(m, r, r)) {
+        if (oz.on && fp64_use_emulated_sliced(m, r, r)) {
             const int64_t r8 = round_up8(r);
             uint16_t *qhs;
             int *eqh;

@@ -499,6 +499,11 @@ cudaError_t launch_store(const SimtPlan &pl, int64_t M, int64_t N, int64_t K, do
     return cudaGetLastError();
 }
 
+// the share of a product's multiply-adds that a triangular result or operand leaves
+inline double needed_share(const GemmExtra &x) {
+    return (x.upper_only ? 0.5 : 1.0) * (x.a_upper && x.b_upper ? 1.0 / 6.0 : x.a_upper || x.b_upper ? 0.5 : 1.0);
+}
+
 template <typename TA, typename TB, typename TC, typename Acc, bool TRA, bool TRB>
 cudaError_t launch(int64_t M, int64_t N, int64_t K, double alpha, const TA *A, int64_t lda,
                    const TB *B, int64_t ldb, double beta, TC *C, int64_t ldc, const GemmExtra &x,
@@ -506,10 +511,7 @@ cudaError_t launch(int64_t M, int64_t N, int64_t K, double alpha, const TA *A, i
 {
     const int flags = (x.upper_only ? F_UPPER_ONLY : 0) | (x.a_upper ? F_A_UPPER : 0) |
                       (x.b_upper ? F_B_UPPER : 0);
-    double frac = 1.0;
-    if (x.upper_only) frac *= 0.5;
-    if (x.a_upper && x.b_upper) frac /= 6.0;
-    else if (x.a_upper || x.b_upper) frac *= 0.5;
+    const double frac = needed_share(x);
     const double flops = 2.0 * (double)M * (double)N * (double)K * frac;
     double bytes = (double)sizeof(TA) * M * K + (double)sizeof(TB) * K * N + (double)sizeof(TC) * M * N;
     if (beta != 0.0 || x.epilogue == EPI_ERR) bytes += (double)sizeof(TC) * M * N;
@@ -544,20 +546,41 @@ cudaError_t launch(int64_t M, int64_t N, int64_t K, double alpha, const TA *A, i
 int64_t gemm_err_ctas(int64_t M, int64_t N) { return ((M + BM - 1) / BM) * ((N + BN - 1) / BN); }
 
 // Large FP64 products go to the tensor-core emulation (oz_gemm.cu) unless
-// EOD_FP64_GEMM=simt; products below 2^25 multiply-adds stay on the SIMT
-// kernel, whose launch and slicing overheads are smaller there.  A skinny
-// side (a few columns) does not exclude the emulation: the SIMT tiles waste
-// as much, and FP64 issue is what they are short of.
-bool fp64_use_emulated(int64_t M, int64_t N, int64_t K) {
+// EOD_FP64_GEMM=simt; small ones stay on the SIMT kernel, whose launch and
+// slicing overheads are smaller there.  A skinny side (a few columns) does not
+// exclude the emulation: the SIMT tiles waste as much, and FP64 issue is what
+// they are short of.  Where the line lies depends on what has to be sliced.
+// SIMT against the emulation with the slicing of both operands, and without
+// that of the first, us (products of the two halves alike):
+//   96 x 96 x 2048      46 /  33 / 26     2048 x 96 x 96      40 / 41 / 27
+//   64 x 64 x 4000      41 /  46 / 35     4000 x 64 x 64      34 / 38 / 25
+//   512 x 256 x 64      22 /  29 / 24     1000 x 32 x 1000    72 / 50 / 26
+//   256 x 256 x 256     39 /  44 / 24     512 x 32 x 384      26 / 40 / 22
+//   1000 x 104 x 1000  200 /  53 / 28     2048 x 128 x 128    65 / 42 / 27
+// Keeping slices of A and Q costs two passes over A and two small launches per
+// block.  Whole factorisations in blocks of 32 without / with them: 716 x 716,
+// rank 13 489 / 514 us, rank 102 1441 / 1376; 620 x 900, rank 20 568 / 575;
+// 800 x 800, rank 30 660 / 607; 1000 x 1000, rank 30 728 / 624.
+static int fp64_mode() {   // 0 SIMT always, 1 by size, 2 emulation always
     static const int mode = [] {
         const char *v = std::getenv("EOD_FP64_GEMM");
         if (v && std::strcmp(v, "simt") == 0) return 0;
         if (v && std::strcmp(v, "emulated") == 0) return 2;
         return 1;
     }();
-    if (mode == 0) return false;
-    if (mode == 2) return M >= 1 && N >= 1 && K >= 1;
-    return (double)M * (double)N * (double)K >= 33554432.0 && K >= 8 && (M >= 128 || N >= 128);
+    return mode;
+}
+static bool fp64_emulate(int64_t M, int64_t N, int64_t K, double least, int64_t side) {
+    if (fp64_mode() != 1) return fp64_mode() == 2 && M >= 1 && N >= 1 && K >= 1;
+    return (double)M * (double)N * (double)K >= least && K >= 8 && (M >= side || N >= side);
+}
+bool fp64_use_emulated(int64_t M, int64_t N, int64_t K) { return fp64_emulate(M, N, K, 33554432.0, 128); }
+bool fp64_use_emulated_sliced(int64_t M, int64_t N, int64_t K) { return fp64_emulate(M, N, K, 1.2e7, 64); }
+bool fp64_keep_slices(int64_t m, int64_t k, int64_t n) { return fp64_emulate(m, k, n, 1.9e7, 128); }
+// any product, both operands to be sliced; frac of its multiply-adds are
+// needed (triangular operands or result), the share the SIMT kernel pays for
+static bool fp64_emulate_product(int64_t M, int64_t N, int64_t K, double frac) {
+    return fp64_use_emulated(M, N, K) || fp64_emulate(M, N, K, 2.1e7 / frac, 64);
 }
 
 // Large FP32 products go to the emulation with four digits (oz_gemm.cu), whose
@@ -585,7 +608,7 @@ cudaError_t gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha
 {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (std::is_same<TA, double>::value && std::is_same<TB, double>::value && std::is_same<TC, double>::value &&
-        ws && ws->err_flag && K > 0 && fp64_use_emulated(M, N, K))
+        ws && ws->err_flag && K > 0 && fp64_emulate_product(M, N, K, needed_share(x)))
         return oz_gemm(ta, tb, M, N, K, alpha, (const double *)A, lda, (const double *)B, ldb, beta, (double *)C,
                        ldc, x, ws->err_flag, s);
     // large FP32 products: the same emulation, rounded once to FP32
