@@ -348,25 +348,53 @@ __global__ void split_norm_kernel(const float *__restrict__ X, int64_t rows, int
     const int64_t tasks = nch * cols;
     int bad = 0;
     float sacc = 0.f, cacc = 0.f;
+    // Four neighbouring rows to a thread where every column starts on 16 bytes (8
+    // in the outputs): one 16-byte load and 8-byte stores.  Bound by HBM: 262144 x
+    // 224 in three terms moves 587 MB (86 us at the copy rate); 167 us with
+    // 4-byte loads and 2-byte stores, and the whole call fell from 1752 to 1678 us.
+    const bool vec = ((ldx | ldo) & 3) == 0 && ((uintptr_t)X & 15) == 0 &&
+                     (((uintptr_t)hi | (uintptr_t)lo | (uintptr_t)x3) & 7) == 0;
+    const int64_t mine = vec ? 4 : 1, step = vec ? 1 : (int64_t)blockDim.x;
     for (int64_t t = blockIdx.x; t < tasks; t += gridDim.x) {
-        const int64_t j = t / nch, i0 = (t - j * nch) * chunk;
+        const int64_t j = t / nch, i0 = (t - j * nch) * chunk + mine * threadIdx.x;
+        const bool whole = vec && i0 + 4 <= rows;
+        float x[U];
+        if (whole) {
+            const float4 v = *(const float4 *)(X + i0 + j * ldx);
+            x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) x[u] = i0 + u * step < rows ? X[i0 + u * step + j * ldx] : 0.f;
+        }
+        __nv_bfloat16 h[U], l[U], r[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t i = i0 + u * (int64_t)blockDim.x + threadIdx.x;
-            if (i < rows) {
-                const float x = X[i + j * ldx];
-                bad |= ((__float_as_uint(x) >> 23) & 0xff) == 0xff;
-                const float pr = x * x;
-                const float er = fmaf(x, x, -pr);
-                const float tt = sacc + pr;
-                const float z = tt - sacc;
-                cacc += ((sacc - (tt - z)) + (pr - z)) + er;
-                sacc = tt;
-                __nv_bfloat16 h, l;
-                split_bf16(x, h, l);
-                hi[i + j * ldo] = h;
-                lo[i + j * ldo] = l;
-                if (x3) x3[i + j * ldo] = __float2bfloat16_rn((x - __bfloat162float(h)) - __bfloat162float(l));
+            bad |= ((__float_as_uint(x[u]) >> 23) & 0xff) == 0xff;
+            const float pr = x[u] * x[u];
+            const float er = fmaf(x[u], x[u], -pr);
+            const float tt = sacc + pr;
+            const float z = tt - sacc;
+            cacc += ((sacc - (tt - z)) + (pr - z)) + er;
+            sacc = tt;
+            split_bf16(x[u], h[u], l[u]);
+            r[u] = __float2bfloat16_rn((x[u] - __bfloat162float(h[u])) - __bfloat162float(l[u]));
+        }
+        if (whole) {
+            auto put = [&](__nv_bfloat16 *o, const __nv_bfloat16 *q) {
+                __nv_bfloat162 w[2] = {__nv_bfloat162(q[0], q[1]), __nv_bfloat162(q[2], q[3])};
+                *(uint2 *)(o + i0 + j * ldo) = *(const uint2 *)w;
+            };
+            put(hi, h);
+            put(lo, l);
+            if (x3) put(x3, r);
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t i = i0 + u * step;
+                if (i >= rows) continue;
+                hi[i + j * ldo] = h[u];
+                lo[i + j * ldo] = l[u];
+                if (x3) x3[i + j * ldo] = r[u];
             }
         }
     }
