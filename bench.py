@@ -236,7 +236,8 @@ KIND_SOURCES = {
     "batch": ["paper_2506_22713_gb300/csrc/batch.cu", "paper_2506_22713_gb300/csrc/chol_leaf.cuh"],
     "oz_gemm": ["paper_2506_22713_gb300/csrc/oz_gemm.cu", "paper_2506_22713_gb300/csrc/tc_ptx.cuh"],
     "tc_gemm": ["paper_2506_22713_gb300/csrc/tc_gemm.cu", "paper_2506_22713_gb300/csrc/tc_ptx.cuh"],
-    "chol": ["paper_2506_22713_gb300/csrc/chol.cu", "paper_2506_22713_gb300/csrc/chol_leaf.cuh"],
+    "chol": ["paper_2506_22713_gb300/csrc/chol.cu", "paper_2506_22713_gb300/csrc/chol_block.cuh",
+             "paper_2506_22713_gb300/csrc/chol_leaf.cuh"],
     "gemm_simt": ["paper_2506_22713_gb300/csrc/gemm_simt.cu"],
     "gemm_simt_f32": ["paper_2506_22713_gb300/csrc/gemm_simt.cu", "paper_2506_22713_gb300/csrc/gram.cu"],
     "stream": ["paper_2506_22713_gb300/csrc/stream_kernels.cu"],
