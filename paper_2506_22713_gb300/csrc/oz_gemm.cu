@@ -635,14 +635,17 @@ __device__ __forceinline__ void digits(float x, int er, __nv_bfloat16 q[NS], boo
 // k (two neighbouring k per lane, one 4-byte store per slice).
 // The row exponents come from the nsplit partial ones of rowexp_kernel (the
 // blocks of the first K column also store them in e_out for the product), or
-// every row takes fixed_e when ep is null.
+// every row takes fixed_e when ep is null.  The tiles are numbered along
+// grid.x, k first: rows or k alone may need more than the 65535 blocks that the
+// other grid dimensions hold (2.1 million rows, 4.2 million k).
 template <typename TX, int NS>
 __global__ void __launch_bounds__(256) slice_kernel(const TX *__restrict__ X, int64_t R, int64_t K, int64_t sr, int64_t sk,
                              int tri, const int *__restrict__ ep, int nsplit, int *__restrict__ e_out, int fixed_e,
                              __nv_bfloat16 *__restrict__ out, int64_t ldk, int64_t slice_stride, int *nonfinite) {
     __shared__ TX tile[32][65];
     __shared__ int erow[32];
-    const int64_t r0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * 64;
+    const unsigned kt = (unsigned)((K + 63) / 64);
+    const int64_t r0 = (int64_t)(blockIdx.x / kt) * 32, k0 = (int64_t)(blockIdx.x % kt) * 64;
     const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
     if (ty == 0) {
         const int64_t r = r0 + tx;
@@ -650,7 +653,7 @@ __global__ void __launch_bounds__(256) slice_kernel(const TX *__restrict__ X, in
         if (ep && r < R) {
             er = kExpZero;
             for (int z = 0; z < nsplit; ++z) er = max(er, ep[(int64_t)z * R + r]);
-            if (blockIdx.x == 0 && e_out) e_out[r] = er;
+            if (k0 == 0 && e_out) e_out[r] = er;
         }
         erow[tx] = er;
     }
@@ -816,8 +819,8 @@ cudaError_t slice_into(const TX *X, int64_t R, int64_t K, int64_t sr, int64_t sk
         }
     }
     count_launch();
-    dim3 grid((unsigned)((K + 63) / 64), (unsigned)((R + 31) / 32));
-    slice_kernel<TX, NS><<<grid, dim3(32, 8), 0, s>>>(X, R, K, sr, sk, tri, ep, (int)ksplit,
+    const int64_t tiles = ((K + 63) / 64) * ((R + 31) / 32);
+    slice_kernel<TX, NS><<<(unsigned)tiles, dim3(32, 8), 0, s>>>(X, R, K, sr, sk, tri, ep, (int)ksplit,
                                                        (ep && ep != e) ? e : nullptr, fixed_e, q, ldk, slice_stride,
                                                        nonfinite);
     cudaError_t le = cudaGetLastError();
