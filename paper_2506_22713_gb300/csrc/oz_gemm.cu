@@ -9,10 +9,8 @@
 // Products of digits are integers of magnitude <= 2^14.  Pairs (s, t) with
 // s + t < NS are grouped by g = s + t (weight 2^(-14 - 8g)); group g holds
 // g + 1 pairs, so over a K chunk of 256 the sums of groups 0-3 are at most
-// 4 * 256 * 2^14 = 2^24 and the tensor core's FP32 accumulation of them is
-// exact.  A later group's sum passes 2^24 only where nearly all its digits are
-// extreme and of one sign, so that the chunk's result is nearly 256 row x
-// column scales; what its rounding then loses is below 2^-49 of that result.
+// 4 * 256 * 2^14 = 2^24, over one of 128 those of the groups above at most
+// 8 * 128 * 2^14 = 2^24, and the tensor core's FP32 accumulation is exact.
 // After each chunk the epilogue warps read the group
 // sums from TMEM as integers and add them to two int64 accumulators per
 // entry (groups 0-3 in units of 2^-38, the others in units of the last
@@ -35,8 +33,9 @@
 // lie one after another in shared memory and the groups s + t in TMEM, so the A
 // rows are read once for up to four slices.  For NS > 4 the products of groups
 // 0-3 come first in every K block, then the others, and the two halves of TMEM
-// are handed over apart: the lower is drained while the chunk's last upper
-// products run, the upper while the next chunk's first lower ones do.
+// are handed over apart: the lower every four K blocks, drained while their last
+// upper products run, the upper every two, drained while the next block's lower
+// ones do.
 // Warp 0: TMA producer, warp 1: MMA issuer, warps 2-17: drain and epilogue
 // (four per TMEM lane quarter, 16 columns each).  All waits are bounded
 // (EOD_ETIMEOUT on expiry).
@@ -56,6 +55,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 namespace eod {
 namespace oz {
@@ -63,7 +63,10 @@ namespace oz {
 using namespace eod::tc;
 
 constexpr int BM = 128, BN = 64, BK = 64;
-constexpr int KCH = 4;                // K blocks per chunk (256)
+constexpr int KCH = 4;                // K blocks per chunk of groups 0-3 (256 terms)
+constexpr int KCH_UPPER = 2;          // and of the groups above (128), which hold up to eight pairs
+static_assert(4 * KCH * BK * 16384 <= 1 << 24 && kOzSlicesFine * KCH_UPPER * BK * 16384 <= 1 << 24 && KCH == 2 * KCH_UPPER,
+              "the group sums stay exact in FP32");
 constexpr int UMMA_K = 16;            // K per tcgen05.mma kind::f16
 constexpr int A_TILE = BM * BK * 2;   // 16 KB: one slice
 constexpr int B_TILE = BN * BK * 2;   // 8 KB
@@ -285,10 +288,6 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         for (int64_t step = 0; ok && w.at(p, step); ++step) {
         const int64_t nkb = w.kb1 - w.kb0;
         for (int64_t q = 0; q < nkb && ok; ++q) {
-            const bool first = (q % KCH) == 0, last = q % KCH == KCH - 1 || q == nkb - 1;
-            const int64_t chunk = chunk0 + q / KCH;
-            const int buf = NBUF > 1 ? (int)(chunk % NBUF) : 0;
-            const uint32_t tacc = tmem + (uint32_t)buf * BUF_COLS;
             const int sb = (int)(ib % BSTAGES);
             ok = warp_wait(&fullB[sb], (uint32_t)((ib / BSTAGES) & 1));
             if (!ok) break;
@@ -296,6 +295,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
             if (__any_sync(0xffffffffu, *(volatile int *)abort_sh != 0)) ok = false;
 #pragma unroll
             for (int h = 0; h < HALVES; ++h) {
+                const int len = h == 0 ? KCH : KCH_UPPER;
+                const bool first = q % len == 0, last = q % len == len - 1 || q == nkb - 1;
+                const int64_t chunk = chunk0 + q / len;   // (chunk0 = 0 with two halves: one tile per CTA)
+                const int buf = NBUF > 1 ? (int)(chunk % NBUF) : 0;
+                const uint32_t tacc = tmem + (uint32_t)buf * BUF_COLS;
                 // the accumulators of this half, once the chunk before has been drained
                 if (first && ok && chunk >= NBUF)
                     ok = warp_wait(&tmem_empty[buf + h], (uint32_t)((chunk / NBUF - 1) & 1));
@@ -358,47 +362,57 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
         const int ecol = p.eb && n0 + c0 + lane < p.N ? max(p.eb[n0 + c0 + lane], -1100) : p.eb_fixed;
         // Per chunk the FP32 group sums (integers) are added to two int64
         // accumulators, groups 0-3 in base 256 (unit 2^-38 of the row x column
-        // scale, |per chunk| < 2^49) and the others (unit 2^(-14 - 8 (NS - 1)),
-        // < 2^50): exact, with no FP64 instruction in the drain.
+        // scale, |per chunk| < 2^47) and the others (unit 2^(-14 - 8 (NS - 1)),
+        // < 2^49): exact, with no FP64 instruction in the drain.
         // (NS = 4: the first accumulator alone.)
         long long acch[ECOLS], accl[ECOLS];
 #pragma unroll
         for (int j = 0; j < ECOLS; ++j) acch[j] = accl[j] = 0;
-        for (int64_t c = chunk0; c < chunk0 + nchunks; ++c) {
+        // chunk c of half h from TMEM into the accumulators; false once a wait ran out
+        auto drain = [&](auto half, int64_t c) -> bool {
+            constexpr int h = decltype(half)::value, g0 = h == 0 ? 0 : 4, ng = h == 0 ? 4 : NG - 4;
             const int buf = NBUF > 1 ? (int)(c % NBUF) : 0;
+            const bool full =
+                __all_sync(0xffffffffu, mbar_wait(&tmem_full[buf + h], (uint32_t)((c / NBUF) & 1)) ? 1 : 0) != 0;
+            if (!full || *(volatile int *)abort_sh) return false;
+            tc_fence_after();
+            // 4 columns at a time: the groups' loads are in flight together
 #pragma unroll
-            for (int h = 0; h < HALVES; ++h) {
-                constexpr int H0 = 4;
-                ok = __all_sync(0xffffffffu, mbar_wait(&tmem_full[buf + h], (uint32_t)((c / NBUF) & 1)) ? 1 : 0) != 0;
-                if (!ok || *(volatile int *)abort_sh) { ok = false; break; }
-                tc_fence_after();
-                const int g0 = h == 0 ? 0 : H0, ng = h == 0 ? H0 : NG - H0;
-                // 4 columns at a time: the groups' loads are in flight together
+            for (int cc = 0; cc < ECOLS; cc += 4) {
+                uint32_t r[4][4];
 #pragma unroll
-                for (int cc = 0; cc < ECOLS; cc += 4) {
-                    uint32_t r[4][4];
+                for (int g = 0; g < ng; ++g)
+                    tmem_ld4_nowait(tmem + ((uint32_t)(32 * qtr) << 16) + (uint32_t)buf * BUF_COLS +
+                                        (uint32_t)((g0 + g) * BN + c0 + cc),
+                                    r[g]);
+                tmem_wait_ld();
 #pragma unroll
-                    for (int g = 0; g < ng; ++g)
-                        tmem_ld4_nowait(tmem + ((uint32_t)(32 * qtr) << 16) + (uint32_t)buf * BUF_COLS +
-                                            (uint32_t)((g0 + g) * BN + c0 + cc),
-                                        r[g]);
-                    tmem_wait_ld();
+                for (int j = 0; j < 4; ++j) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-#pragma unroll
-                        for (int g = 0; g < ng; ++g) {
-                            const int iv = __float2int_rn(__uint_as_float(r[g][j]));
-                            if (h == 0) acch[cc + j] = mad_wide(iv, 1 << (8 * (3 - g)), acch[cc + j]);
-                            else accl[cc + j] = mad_wide(iv, 1 << (8 * (NG - 1 - H0 - g)), accl[cc + j]);
-                        }
+                    for (int g = 0; g < ng; ++g) {
+                        const int iv = __float2int_rn(__uint_as_float(r[g][j]));
+                        if (h == 0) acch[cc + j] = mad_wide(iv, 1 << (8 * (3 - g)), acch[cc + j]);
+                        else accl[cc + j] = mad_wide(iv, 1 << (8 * (NG - 5 - g)), accl[cc + j]);
                     }
                 }
-                tc_fence_before();
-                mbar_arrive(&tmem_empty[buf + h]);
             }
-            if (!ok) break;
+            tc_fence_before();
+            mbar_arrive(&tmem_empty[buf + h]);
+            return true;
+        };
+        // in the order in which the issuer hands them over
+        using Lower = std::integral_constant<int, 0>;
+        using Upper = std::integral_constant<int, HALVES - 1>;
+        if constexpr (HALVES == 1) {
+            for (int64_t c = 0; c < nchunks && ok; ++c) ok = drain(Lower(), chunk0 + c);
+            chunk0 += nchunks;
+        } else {
+            const int64_t nupper = (w.kb1 - w.kb0 + KCH_UPPER - 1) / KCH_UPPER;
+            for (int64_t u = 0; u < nupper && ok; ++u) {
+                if ((u & 1) || u == nupper - 1) ok = drain(Lower(), u >> 1);
+                if (ok) ok = drain(Upper(), u);
+            }
         }
-        chunk0 += nchunks;
         if (!ok) {
             atomicExch(p.err_flag, 1);
             break;
