@@ -216,7 +216,7 @@ constexpr int kOzSlicesF32 = 4;    // FP32 data and result (oz_gemm_f32)
 
 // whether gemm<double,...> sends an M x N x K product to oz_gemm
 bool fp64_use_emulated(int64_t M, int64_t N, int64_t K);
-bool fp64_use_emulated_sliced(int64_t M, int64_t N, int64_t K);   // one operand's slices are there
+bool fp64_use_emulated_sliced(int64_t M, int64_t N, int64_t K);   // one operand's slices, of its rows' own exponents, are there
 bool fp64_keep_slices(int64_t m, int64_t k, int64_t n);            // A (m x n) in blocks of k: slices of A and Q kept
 // whether gemm<float,...> sends an M x N x K product to oz_gemm_f32
 bool fp32_use_emulated(int64_t M, int64_t N, int64_t K);

@@ -537,7 +537,12 @@ struct Result {
 // orientations (sliced once), the basis Q in both orientations (extended as
 // columns are appended: per-column exponents for Q^T, the fixed exponent 1
 // for Q, whose entries are at most 1 in magnitude), and a buffer for the
-// small operand of each product.
+// small operand of each product.  The fixed exponent costs accuracy: a dense
+// Q's entries are near m^-1/2, rows of small scale far below, and what a digit
+// holds is relative to 2 (Q S, m = 1500, 600 columns: 3.8e-15 relative, FP64
+// FMAs 8.2e-16, digits of each row's own exponent 2.4e-16).  So Q's row slices
+// serve only the products of 2^25 multiply-adds and more; smaller ones go
+// through gemm(), which slices rows at their own exponents or uses FMAs.
 struct OzCache {
     bool on = false;
     void *Arow = nullptr, *Acol = nullptr, *Qc = nullptr, *Qr = nullptr, *Bt = nullptr;
@@ -696,7 +701,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             e = gemm<T, T, T, T>(true, false, nq, wdt, m, 1.0, Qq, m, Yc, m, 0.0, Sb, cap, ex, w, st);
         }
         if (e != cudaSuccess) return e;
-        if (oz.on && fp64_use_emulated_sliced(m, wdt, nq) && q0 % 8 == 0) {
+        if (oz.on && fp64_use_emulated(m, wdt, nq) && q0 % 8 == 0) {
             OzOperand bo;
             e = oz_small_to(Sb, wdt, nq, cap, 1, bt, ebt, st, bo);
             if (e != cudaSuccess) return e;
@@ -1018,7 +1023,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
             const int64_t nct = gemm_err_ctas(m, n);
             double *part;
             EOD_TRY(ar.get(&part, (size_t)nct));
-            const bool emulated = oz.on && fp64_use_emulated_sliced(m, n, r);
+            const bool emulated = oz.on && fp64_use_emulated(m, n, r);
             uint16_t *cts = nullptr;
             int *ects = nullptr;
             const int64_t r8 = round_up8(r);
@@ -1068,7 +1073,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     }
     // U = Q Qh
     auto form_u = [&]() -> eod_status {
-        if (oz.on && fp64_use_emulated_sliced(m, r, r)) {
+        if (oz.on && fp64_use_emulated(m, r, r)) {
             const int64_t r8 = round_up8(r);
             uint16_t *qhs;
             int *eqh;
