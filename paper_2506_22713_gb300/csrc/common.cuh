@@ -109,6 +109,7 @@ struct Scratch {
 // when the call returns unless handed over with keep().
 // --------------------------------------------------------------------------
 extern int g_fail_alloc_after;   // test hook: n-th allocation from now fails
+inline bool fail_this_alloc() { return g_fail_alloc_after > 0 && --g_fail_alloc_after == 0; }
 
 // Stream-ordered allocation from the library's own memory pool on the
 // current device.  The pool keeps up to 64 GiB of freed blocks mapped, so the
@@ -125,9 +126,7 @@ struct Arena {
     eod_status get(T **p, size_t count) {
         *p = nullptr;
         if (count == 0) count = 1;
-        if (g_fail_alloc_after > 0) {
-            if (--g_fail_alloc_after == 0) return EOD_ENOMEM;
-        }
+        if (fail_this_alloc()) return EOD_ENOMEM;
         void *q = nullptr;
         cudaError_t e = lib_malloc_async(&q, sizeof(T) * count, s);
         if (e != cudaSuccess) {

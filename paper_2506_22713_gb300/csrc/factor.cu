@@ -1276,9 +1276,8 @@ static eod_status reconstruct_impl(const eod_factors *f, T *Ahat, int64_t ld, cu
     };
     if (std::is_same<T, double>::value ? fp64_use_emulated(m, n, r) : fp32_use_emulated(m, n, r)) {
         // The larger of the two products (or both) on the tensor cores.  The
-        // emulation takes non-finite entries for
-        // zero, and it needs room for the operands' slices: where either
-        // happens, the DFMA products below give the result instead.
+        // emulation takes non-finite entries for zero: where any were sliced,
+        // the FMA products below give the result instead.
         int *flags;   // [0] a wait ran out, [1] a non-finite entry was sliced
         EOD_TRY(ar.get(&flags, 2));
         EOD_CU(cudaMemsetAsync(flags, 0, sizeof(int) * 2, s));
@@ -1288,17 +1287,12 @@ static eod_status reconstruct_impl(const eod_factors *f, T *Ahat, int64_t ld, cu
         const cudaError_t e = products();
         ws.err_flag = nullptr;
         ex.nonfinite = bu.nonfinite = nullptr;
-        if (e == cudaSuccess) {
-            int h[2] = {0, 0};
-            EOD_CU(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s));
-            EOD_CU(cudaStreamSynchronize(s));
-            if (h[0]) return EOD_ETIMEOUT;
-            if (!h[1]) return EOD_OK;
-        } else if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-        } else {
-            return cuda_status(e);
-        }
+        EOD_CU(e);
+        int h[2] = {0, 0};
+        EOD_CU(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s));
+        EOD_CU(cudaStreamSynchronize(s));
+        if (h[0]) return EOD_ETIMEOUT;
+        if (!h[1]) return EOD_OK;
     }
     EOD_CU(products());
     return EOD_OK;
@@ -1348,7 +1342,7 @@ eod_status eod_abe_factor_host(const void *A_host, int64_t m, int64_t n, int64_t
     cudaStream_t s = (cudaStream_t)o.stream;
     const size_t es = o.a_dtype == EOD_F64 ? 8 : 4;
     void *Ad = nullptr;
-    if (g_fail_alloc_after > 0 && --g_fail_alloc_after == 0) return EOD_ENOMEM;
+    if (fail_this_alloc()) return EOD_ENOMEM;
     if (lib_malloc_async(&Ad, es * (size_t)m * n, s) != cudaSuccess) { cudaGetLastError(); return EOD_ENOMEM; }
     eod_status st = EOD_OK;
     if (cudaMemcpy2DAsync(Ad, es * m, A_host, es * lda, es * m, n, cudaMemcpyHostToDevice, s) != cudaSuccess)

@@ -608,14 +608,20 @@ cudaError_t gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha
 {
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (std::is_same<TA, double>::value && std::is_same<TB, double>::value && std::is_same<TC, double>::value &&
-        ws && ws->err_flag && K > 0 && fp64_emulate_product(M, N, K, needed_share(x)))
-        return oz_gemm(ta, tb, M, N, K, alpha, (const double *)A, lda, (const double *)B, ldb, beta, (double *)C,
-                       ldc, x, ws->err_flag, s);
+        ws && ws->err_flag && K > 0 && fp64_emulate_product(M, N, K, needed_share(x))) {
+        const cudaError_t e = oz_gemm(ta, tb, M, N, K, alpha, (const double *)A, lda, (const double *)B, ldb, beta,
+                                      (double *)C, ldc, x, ws->err_flag, s);
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();   // no room for the slices (up to twice an operand): the FMA kernels need none
+    }
     // large FP32 products: the same emulation, rounded once to FP32
     if (std::is_same<TA, float>::value && std::is_same<TB, float>::value && std::is_same<TC, float>::value &&
-        ws && ws->err_flag && K > 0 && x.epilogue == EPI_STORE && fp32_use_emulated(M, N, K))
-        return oz_gemm_f32(ta, tb, M, N, K, alpha, (const float *)A, lda, (const float *)B, ldb, beta, (float *)C,
-                           ldc, x, ws->err_flag, s);
+        ws && ws->err_flag && K > 0 && x.epilogue == EPI_STORE && fp32_use_emulated(M, N, K)) {
+        const cudaError_t e = oz_gemm_f32(ta, tb, M, N, K, alpha, (const float *)A, lda, (const float *)B, ldb, beta,
+                                          (float *)C, ldc, x, ws->err_flag, s);
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+    }
     // matrix-vector products: op(B) is one column of K contiguous values
     if (N == 1 && !tb && K > 0 && x.epilogue == EPI_STORE && !x.upper_only && !x.a_upper && !x.b_upper && ws)
         return launch_gemv<TA, TB, TC, Acc>(ta, M, K, alpha, A, lda, B, beta, C, ws, s);

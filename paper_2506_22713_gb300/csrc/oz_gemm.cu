@@ -794,6 +794,12 @@ __global__ void split_sum_kernel(const double *__restrict__ part, int S, int64_t
     }
 }
 
+// The emulation's own buffers: without room for them the caller takes the FMA
+// kernels (nothing has been written to C by then).
+cudaError_t room(void **p, size_t bytes, cudaStream_t s) {
+    return fail_this_alloc() ? cudaErrorMemoryAllocation : lib_malloc_async(p, bytes, s);
+}
+
 struct Slices {
     __nv_bfloat16 *q = nullptr;
     int *e = nullptr;
@@ -823,7 +829,7 @@ cudaError_t slice_into(const TX *X, int64_t R, int64_t K, int64_t sr, int64_t sk
         const int64_t kper = (K + ksplit - 1) / ksplit;
         ksplit = (K + kper - 1) / kper;
         ep = e;   // one range: the partial exponents are the exponents
-        if (ksplit > 1) EOD_CUDA_TRY(lib_malloc_async((void **)&ep, sizeof(int) * (size_t)ksplit * R, s));
+        if (ksplit > 1) EOD_CUDA_TRY(room((void **)&ep, sizeof(int) * (size_t)ksplit * R, s));
         count_launch();
         rowexp_kernel<<<dim3((unsigned)rblocks, (unsigned)ksplit), 256, 0, s>>>(X, R, K, sr, sk, kper, tri, ep);
         cudaError_t le = cudaGetLastError();
@@ -847,8 +853,8 @@ cudaError_t make_slices(const TX *X, int64_t R, int64_t K, int64_t sr, int64_t s
                         int tri = 0, int *nonfinite = nullptr) {
     sl.R = R;
     sl.ldk = round_up(K, 8);
-    EOD_CUDA_TRY(lib_malloc_async((void **)&sl.q, sizeof(__nv_bfloat16) * (size_t)NS * R * sl.ldk, s));
-    EOD_CUDA_TRY(lib_malloc_async((void **)&sl.e, sizeof(int) * (size_t)R, s));
+    EOD_CUDA_TRY(room((void **)&sl.q, sizeof(__nv_bfloat16) * (size_t)NS * R * sl.ldk, s));
+    EOD_CUDA_TRY(room((void **)&sl.e, sizeof(int) * (size_t)R, s));
     return slice_into<NS>(X, R, K, sr, sk, sl.q, sl.e, 0, sl.ldk, R * sl.ldk, s, tri, nonfinite);
 }
 
@@ -921,7 +927,7 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
     if constexpr (NS != kOzSlicesF32)
         if (e == cudaSuccess) e = set_smem_once(oz_gemm_kernel<NS, EPI_ERR>, SMEM);
     if (e == cudaSuccess && splits > 1) {
-        e = lib_malloc_async((void **)&part, sizeof(double) * (size_t)splits * M * N, s);
+        e = room((void **)&part, sizeof(double) * (size_t)splits * M * N, s);
         p.C = part;
         p.ldc = M;
         p.split_stride = M * N;
