@@ -154,7 +154,7 @@ struct Arena {
 //   grid would not fill the GPU; the split partials are summed in a fixed
 //   order, so results are deterministic.
 // --------------------------------------------------------------------------
-enum GemmEpilogue { EPI_STORE = 0, EPI_ERR = 1 };
+enum GemmEpilogue { EPI_STORE = 0, EPI_ERR = 1, EPI_COVER = 2 };   // (EPI_COVER: tc_gemm.cuh only)
 
 struct GemmExtra {
     bool upper_only = false;   // only tiles that touch the upper triangle of C
@@ -165,8 +165,7 @@ struct GemmExtra {
     int64_t ldref = 0;
     double *err_partials = nullptr; // EPI_ERR: one double per CTA (gridDim.x*gridDim.y)
     int max_split = 64;
-    bool fine = false;         // emulated FP64: one more slice (see oz_gemm.cu)
-    int *nonfinite = nullptr;  // emulated FP64: set when an operand holds a NaN or an infinity (sliced as zero)
+    const int *skip = nullptr; // emulated products: nothing is computed where this device flag is set
     int force_ts = 0;          // SIMT tile forced by the autotuner's timing hook (0 = plan)
 };
 
@@ -204,17 +203,27 @@ cudaError_t oz_gemm_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64
 cudaError_t oz_gemm_f32(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const float *A, int64_t lda,
                         const float *B, int64_t ldb, double beta, float *C, int64_t ldc, const GemmExtra &x,
                         int *err_flag, cudaStream_t s);
+// A_hat (m x n) = W V^T with W (m x r) = U D, D upper triangular (r x r): both
+// products emulated, or the second alone when W is given (U == nullptr).
+// flags (two zeroed device ints): [0] a bounded wait ran out; [1] A_hat is not
+// to be used, because an operand holds a NaN or an infinity (sliced as zero) or
+// because the digits do not carry every entry to the accuracy of FMAs (see
+// oz_gemm.cu).
+template <typename T>
+cudaError_t oz_decode(const T *U, const T *D, T *W, const T *V, int64_t m, int64_t n, int64_t r, T *A_hat, int64_t ld,
+                      int *flags, cudaStream_t s);
 // slices of op(X) (rows x K, X(r, k) at X[r*sr + k*sk]) into q (ld ldk, slices
 // slice_stride apart); per-row exponents into e, or the fixed exponent when e
 // is null (every |X| must then be below 2^fixed_e)
 cudaError_t oz_slice(const double *X, int64_t rows, int64_t K, int64_t sr, int64_t sk, void *q, int *e,
                      int fixed_e, int64_t ldk, int64_t slice_stride, cudaStream_t s);
 constexpr int kOzSlices = 7;       // the factorisation's products
-constexpr int kOzSlicesFine = 8;   // GemmExtra::fine
+constexpr int kOzSlicesFine = 8;   // A_hat in FP64
 constexpr int kOzSlicesF32 = 4;    // FP32 data and result (oz_gemm_f32)
 
 // whether gemm<double,...> sends an M x N x K product to oz_gemm
 bool fp64_use_emulated(int64_t M, int64_t N, int64_t K);
+bool fp64_emulate_product(int64_t M, int64_t N, int64_t K, double frac);   // frac: its multiply-adds needed
 bool fp64_use_emulated_sliced(int64_t M, int64_t N, int64_t K);   // one operand's slices, of its rows' own exponents, are there
 bool fp64_keep_slices(int64_t m, int64_t k, int64_t n);            // A (m x n) in blocks of k: slices of A and Q kept
 // whether gemm<float,...> sends an M x N x K product to oz_gemm_f32

@@ -1269,32 +1269,36 @@ static eod_status reconstruct_impl(const eod_factors *f, T *Ahat, int64_t ld, cu
     EOD_CU((copy_matrix<double, T>(f->D, r, Dt, r, r, r, false, s)));
     GemmExtra ex, bu;
     bu.b_upper = true;
+    constexpr bool f64 = std::is_same<T, double>::value;
     const T *U = (const T *)f->U, *V = (const T *)f->V;
-    auto products = [&]() -> cudaError_t {
-        const cudaError_t e = gemm<T, T, T, T>(false, false, m, r, r, 1.0, U, m, Dt, r, 0.0, W, m, bu, &ws, s);   // W = U D
-        return e != cudaSuccess ? e : gemm<T, T, T, T>(false, true, m, n, r, 1.0, W, m, V, n, 0.0, Ahat, ld, ex, &ws, s);
-    };
-    if (std::is_same<T, double>::value ? fp64_use_emulated(m, n, r) : fp32_use_emulated(m, n, r)) {
-        // The larger of the two products (or both) on the tensor cores.  The
-        // emulation takes non-finite entries for zero: where any were sliced,
-        // the FMA products below give the result instead.
-        int *flags;   // [0] a wait ran out, [1] a non-finite entry was sliced
+    auto fma_w = [&]() { return gemm<T, T, T, T>(false, false, m, r, r, 1.0, U, m, Dt, r, 0.0, W, m, bu, &ws, s); };   // W = U D
+    bool w_given = false;
+    if (f64 ? fp64_use_emulated(m, n, r) : fp32_use_emulated(m, n, r)) {
+        // On the tensor cores: A_hat = W V^T, and W in FP64 where it is large
+        // (in FP32 FMAs are as fast: 8192 x 455 x 455 85 us against 41 and
+        // 41 of slicing).
+        // Where the digits cannot vouch for every entry, or have no room, the
+        // FMA products below give the result instead.
+        w_given = !(f64 && fp64_emulate_product(m, r, r, 0.5));
+        if (w_given) EOD_CU(fma_w());
+        int *flags;
         EOD_TRY(ar.get(&flags, 2));
         EOD_CU(cudaMemsetAsync(flags, 0, sizeof(int) * 2, s));
-        ws.err_flag = flags;
-        ex.nonfinite = bu.nonfinite = flags + 1;
-        ex.fine = bu.fine = true;
-        const cudaError_t e = products();
-        ws.err_flag = nullptr;
-        ex.nonfinite = bu.nonfinite = nullptr;
-        EOD_CU(e);
-        int h[2] = {0, 0};
-        EOD_CU(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s));
-        EOD_CU(cudaStreamSynchronize(s));
-        if (h[0]) return EOD_ETIMEOUT;
-        if (!h[1]) return EOD_OK;
+        const cudaError_t e = oz_decode<T>(w_given ? nullptr : U, Dt, W, V, m, n, r, Ahat, ld, flags, s);
+        if (e == cudaSuccess) {
+            int h[2] = {0, 0};
+            EOD_CU(cudaMemcpyAsync(h, flags, sizeof(h), cudaMemcpyDeviceToHost, s));
+            EOD_CU(cudaStreamSynchronize(s));
+            if (h[0]) return EOD_ETIMEOUT;
+            if (!h[1]) return EOD_OK;
+        } else if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+        } else {
+            return cuda_status(e);
+        }
     }
-    EOD_CU(products());
+    if (!w_given) EOD_CU(fma_w());
+    EOD_CU((gemm<T, T, T, T>(false, true, m, n, r, 1.0, W, m, V, n, 0.0, Ahat, ld, ex, &ws, s)));   // A_hat = W V^T
     return EOD_OK;
 }
 

@@ -579,7 +579,7 @@ bool fp64_use_emulated_sliced(int64_t M, int64_t N, int64_t K) { return fp64_emu
 bool fp64_keep_slices(int64_t m, int64_t k, int64_t n) { return fp64_emulate(m, k, n, 1.9e7, 128); }
 // any product, both operands to be sliced; frac of its multiply-adds are
 // needed (triangular operands or result), the share the SIMT kernel pays for
-static bool fp64_emulate_product(int64_t M, int64_t N, int64_t K, double frac) {
+bool fp64_emulate_product(int64_t M, int64_t N, int64_t K, double frac) {
     return fp64_use_emulated(M, N, K) || fp64_emulate(M, N, K, 2.1e7 / frac, 64);
 }
 

@@ -24,8 +24,12 @@
 //   own rounding.  Its 4 x 64 accumulator columns fit TMEM twice, so a chunk is
 //   drained while the next is multiplied; with more tiles than SMs a CTA takes
 //   several, its products running ahead of its epilogues.
-//   NS = 8 (36 products): where the result has to be as accurate as FP64 FMAs
-//   whatever the operands' spread (A_hat = U D V^T).
+//   NS = 8 (36 products): A_hat = U D V^T in FP64.
+// These errors are relative to the largest entry of the row times that of the
+// column, not to the entry computed: where an entry's own terms are far smaller
+// (operands graded along k, zeros against the large ones) FMAs are the more
+// accurate.  The factorisations' results are accurate in norm only, so there it
+// is enough; A_hat is checked entry by entry (oz_decode).
 //
 // CTA tile 128 x 64; a K block of 64 stages all NS B slices and streams the
 // NS A slices through a ring; TMEM holds NS x 64 FP32 group accumulators.  An
@@ -106,6 +110,7 @@ struct Params {
     int64_t ldr;
     double *errp;
     int *err_flag;
+    const int *skip;          // nothing is done where this is set (null: always done)
     int upper_only;           // store only entries with row <= col
     int a_tri, b_tri;         // op(A) / op(B) upper triangular: skip their zero K blocks
     int64_t gm, tiles;        // NS = 4: tile rows, and the tiles a CTA strides over (0: one tile per CTA)
@@ -217,6 +222,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) oz_gemm_kernel(const __grid_const
     int *abort_sh = (int *)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (p.skip && *p.skip) return;   // set by earlier kernels of the stream: the same for every thread
     Tile<NS == kOzSlicesF32> w;
     if (!(NS == kOzSlicesF32 && p.tiles > 0) && p.upper_only) {   // every entry of the tile is below the diagonal
         w.at(p, 0);
@@ -899,6 +905,7 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
     p.alpha = alpha;
     p.beta = beta;
     p.err_flag = err_flag;
+    p.skip = x.skip;
     p.R = (const double *)x.ref;
     p.ldr = x.ldref;
     p.errp = x.err_partials;
@@ -990,9 +997,9 @@ cudaError_t gemm_any(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double a
     // op(A)(i, k): rows i, reduction k; op(B)(k, j) seen as rows j
     // a_upper / b_upper: op(A) / op(B) is upper triangular and its zero part
     // is not read, as in the SIMT kernel
-    cudaError_t e = make_slices<NS>(A, M, K, ta ? lda : 1, ta ? 1 : lda, sa, s, x.a_upper ? 1 : 0, x.nonfinite);
+    cudaError_t e = make_slices<NS>(A, M, K, ta ? lda : 1, ta ? 1 : lda, sa, s, x.a_upper ? 1 : 0);
     const bool same = (A == B) && (ta != tb) && (lda == ldb) && (M == N) && !x.a_upper && !x.b_upper;
-    if (e == cudaSuccess && !same) e = make_slices<NS>(B, N, K, tb ? 1 : ldb, tb ? ldb : 1, sb, s, x.b_upper ? 2 : 0, x.nonfinite);
+    if (e == cudaSuccess && !same) e = make_slices<NS>(B, N, K, tb ? 1 : ldb, tb ? ldb : 1, sb, s, x.b_upper ? 2 : 0);
     const Slices &SB = same ? sa : sb;
     if (e == cudaSuccess) {
         OzOperand oa{sa.q, sa.e, 0, sa.ldk, (int64_t)M * sa.ldk};
@@ -1010,9 +1017,6 @@ cudaError_t gemm_any(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double a
 cudaError_t oz_gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A, int64_t lda,
                     const double *B, int64_t ldb, double beta, double *C, int64_t ldc, const GemmExtra &x,
                     int *err_flag, cudaStream_t s) {
-    if (x.fine)
-        return oz::gemm_any<kOzSlicesFine, double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, nullptr, ldc, x,
-                                                   err_flag, s);
     return oz::gemm_any<kOzSlices, double>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, nullptr, ldc, x, err_flag, s);
 }
 
@@ -1024,6 +1028,157 @@ cudaError_t oz_gemm_f32(bool ta, bool tb, int64_t M, int64_t N, int64_t K, doubl
     if (x.epilogue != EPI_STORE) return cudaErrorInvalidValue;
     return oz::gemm_any<kOzSlicesF32, float>(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, nullptr, C, ldc, x, err_flag, s);
 }
+
+namespace oz {
+
+// What the check of oz_decode takes of the sliced operands W (R_w rows, then V's),
+// one warp per row: the entries' magnitudes in BF16, rounded towards zero from
+// |256 q_0 + q_1| - 1 <= 2^15 |x| / 2^e, and the row's part of what each entry of
+// A_hat needs (oz_decode): rows of W scale (1, 2^(eu + E - e)), eu the exponent
+// of U's row, E the largest of D's nd columns' ed; rows of V (1, sum over l of
+// 2^(ed_l - E) |x_l| / 2^e).  With nd = 0 (W given) the second part is zero.  A
+// row of zeros needs nothing, unless W's came out of a U that is not zero: then
+// no entry is vouched for.  (Reads and writes 6 bytes an entry; 2 x 8192 rows of
+// 455: 15 us.)
+__global__ void __launch_bounds__(256) cover_rows_kernel(const __nv_bfloat16 *__restrict__ qw,
+                                                         const __nv_bfloat16 *__restrict__ qv, int64_t R_w, int64_t R,
+                                                         int64_t K, int64_t ldk, const int *__restrict__ ew,
+                                                         const int *__restrict__ ev, const int *__restrict__ eu,
+                                                         const int *__restrict__ ed, int64_t nd, float scale,
+                                                         __nv_bfloat16 *__restrict__ mag, float2 *__restrict__ need) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (row >= R) return;
+    const bool of_w = row < R_w;
+    const int64_t at = of_w ? row : row - R_w;
+    const __nv_bfloat16 *q = (of_w ? qw : qv) + at * ldk;
+    const int64_t stride = (of_w ? R_w : R - R_w) * ldk;
+    int E = kExpZero;
+    for (int64_t l = lane; l < nd; l += 32) E = max(E, ed[l]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) E = max(E, __shfl_xor_sync(0xffffffffu, E, o));
+    float sum = 0.f;
+    for (int64_t k = 8 * lane; k < K; k += 256) {   // (ldk is a multiple of 8; what lies beyond K is not used)
+        union Eight {
+            uint4 v;
+            __nv_bfloat16 x[8];
+        } a, b, m;
+        a.v = *(const uint4 *)(q + k);
+        b.v = *(const uint4 *)(q + stride + k);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float h = fabsf(fmaf(256.f, __bfloat162float(a.x[j]), __bfloat162float(b.x[j])));
+            m.x[j] = __float2bfloat16_rz(fmaxf(h - 1.f, 0.f));
+            if (nd && !of_w && k + j < K) sum = fmaf(h + 1.f, exp2f((float)max(ed[k + j] - E, -200)), sum);
+        }
+        *(uint4 *)(mag + row * ldk + k) = m.v;
+    }
+    sum = warp_sum(sum);
+    if (lane) return;
+    float2 n = make_float2(of_w ? scale : 1.f, 0.f);
+    const int er = of_w ? ew[at] : ev[at], er_u = of_w && nd ? eu[at] : kExpZero;
+    if (er == kExpZero) n.x = er_u != kExpZero ? __int_as_float(0x7f800000) : 0.f;
+    else if (nd) n.y = !of_w ? ldexpf(sum, -15) : er_u == kExpZero ? 0.f : scale * exp2f((float)max(er_u + E - er, -126));
+    need[row] = n;
+}
+
+// The rounding of the digits, and the pairs left out (s + t >= NS), take at
+// most (NS + 1.1) 2^(-8 NS) of the row x column scales per term.
+template <int NS> constexpr double kTermLoss = NS == 8 ? 9.1 / 18446744073709551616.0 : 5.1 / 4294967296.0;
+
+// A_hat = W V^T through the emulation, W = U D as well if U is given, but only
+// if no entry loses anything against FMAs.  Those guarantee 2 r u S(i, j) (and
+// the result's rounding), S = |W| |V|^T; the digits, with a = eta r, eta =
+// kTermLoss, e the row exponents and e_U, e_D those of U's rows and D's
+// columns,
+//   a 2^(e_W(i) + e_V(j))  +  a 2^e_U(i) sum over l of 2^e_D(l) |V(j, l)|,
+// the second for W's own error.  So S(i, j) has to be eta / 2u times the sum of
+// the two powers: 1/450 of it in FP64, 1/100 in FP32.  S is bounded from below by a
+// product of the magnitudes' first eight bits on the tensor cores, compared in
+// its epilogue (both kernels: 28 of 415 us in FP64 at 2048 x 2048 x 600, 100 of
+// 884 in FP32 at 8192 x 8192 x 455); where any entry falls short, flags[1] is
+// set and the large product is not run.
+// Dense factors pass (the least entry of 3000 x 3000 by a factor of 5 with D's
+// diagonal falling as 1/l, of 66 with the FP64 form's test factors); rows of V
+// with zeros against W's large entries do not, nor all of a diagonal that falls
+// as fast as 1/l^2.
+template <typename T>
+cudaError_t decode(const T *U, const T *D, T *W, const T *V, int64_t m, int64_t n, int64_t r, T *A_hat, int64_t ld,
+                   int *flags, cudaStream_t s) {
+    constexpr bool f64 = std::is_same<T, double>::value;
+    constexpr int NS = f64 ? kOzSlicesFine : kOzSlicesF32;
+    Slices su, sd, sw, sv;
+    __nv_bfloat16 *mag = nullptr;
+    float2 *need = nullptr;
+    GemmExtra x;
+    cudaError_t e = cudaSuccess;
+    if (U) {
+        if constexpr (f64) {
+            e = make_slices<NS>(U, m, r, 1, m, su, s, 0, flags + 1);
+            if (e == cudaSuccess) e = make_slices<NS>(D, r, r, r, 1, sd, s, 2, flags + 1);
+            if (e == cudaSuccess) {
+                const OzOperand ou{su.q, su.e, 0, su.ldk, m * su.ldk}, od{sd.q, sd.e, 0, sd.ldk, r * sd.ldk};
+                x.b_upper = true;
+                e = run_ops<NS>(ou, od, m, r, r, 1.0, 0.0, W, m, x, flags, s, nullptr);
+                x.b_upper = false;
+            }
+        } else {
+            e = cudaErrorInvalidValue;
+        }
+    }
+    if (e == cudaSuccess) e = make_slices<NS>(W, m, r, 1, m, sw, s, 0, flags + 1);
+    if (e == cudaSuccess) e = make_slices<NS>(V, n, r, 1, n, sv, s, 0, flags + 1);
+    if (e == cudaSuccess) e = room((void **)&mag, sizeof(__nv_bfloat16) * (size_t)((m + n) * sw.ldk), s);
+    if (e == cudaSuccess) e = room((void **)&need, sizeof(float2) * (size_t)(m + n), s);
+    if (e == cudaSuccess) {
+        ProfScope prof(PROF_STREAM, 0.0, 6.0 * (m + n) * r, s);
+        count_launch();
+        const double u = f64 ? 1.0 / 9007199254740992.0 : 1.0 / 16777216.0;
+        // S in units of 2^-30 of the scales; a fifth more for the FP32 sums
+        const float scale = (float)(1.2 * 1073741824.0 * kTermLoss<NS> / (2.0 * u));
+        cover_rows_kernel<<<(unsigned)((m + n + 7) / 8), 256, 0, s>>>(sw.q, sv.q, m, m + n, r, sw.ldk, sw.e, sv.e, su.e, sd.e,
+                                                                      U ? r : 0, scale, mag, need);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+        TcGemmDesc g;
+        g.M = m;
+        g.N = n;
+        g.K = r;
+        g.a[0] = {mag, r, m, sw.ldk};
+        g.b[0] = {mag + m * sw.ldk, r, n, sv.ldk};
+        g.epilogue = EPI_COVER;
+        g.row_need = need;
+        g.col_need = need + m;
+        g.low = flags + 1;
+        g.err_flag = flags;
+        e = tc_gemm_run(g, nullptr, s);
+    }
+    if (e == cudaSuccess) {
+        const OzOperand ow{sw.q, sw.e, 0, sw.ldk, m * sw.ldk}, ov{sv.q, sv.e, 0, sv.ldk, n * sv.ldk};
+        x.skip = flags + 1;
+        if constexpr (f64) e = run_ops<NS>(ow, ov, m, n, r, 1.0, 0.0, A_hat, ld, x, flags, s, nullptr);
+        else e = run_ops<NS>(ow, ov, m, n, r, 1.0, 0.0, nullptr, ld, x, flags, s, A_hat);
+    }
+    free_slices(su, s);
+    free_slices(sd, s);
+    free_slices(sw, s);
+    free_slices(sv, s);
+    if (mag) cudaFreeAsync(mag, s);
+    if (need) cudaFreeAsync(need, s);
+    return e;
+}
+}  // namespace oz
+
+template <typename T>
+cudaError_t oz_decode(const T *U, const T *D, T *W, const T *V, int64_t m, int64_t n, int64_t r, T *A_hat, int64_t ld,
+                      int *flags, cudaStream_t s) {
+    return oz::decode<T>(U, D, W, V, m, n, r, A_hat, ld, flags, s);
+}
+template cudaError_t oz_decode<double>(const double *, const double *, double *, const double *, int64_t, int64_t, int64_t,
+                                       double *, int64_t, int *, cudaStream_t);
+template cudaError_t oz_decode<float>(const float *, const float *, float *, const float *, int64_t, int64_t, int64_t,
+                                      float *, int64_t, int *, cudaStream_t);
 
 int64_t oz_gemm_err_ctas(int64_t M, int64_t N) { return ((M + oz::BM - 1) / oz::BM) * ((N + oz::BN - 1) / oz::BN); }
 

@@ -100,6 +100,8 @@ struct Params {
     const float *R;        // EPI_ERR: reference
     int64_t ldr;
     double *errp;          // EPI_ERR: one partial per CTA
+    const float2 *row_need, *col_need;   // EPI_COVER
+    int *low;
     int *err_flag;         // timeout flag
 };
 
@@ -108,15 +110,16 @@ struct Cfg {
     static constexpr int A_BYTES = BM * BK * 2;          // 16 KB
     static constexpr int B_BYTES = BN_ * BK * 2;
     static constexpr int STAGE = A_BYTES + B_BYTES;
-    // The fused error epilogue reads a tile of A after the MMAs; two stages
-    // leave room for a second CTA on the SM, whose MMAs overlap that read.
-    static constexpr int STAGES = (EPI == EPI_ERR) ? 2 : ((BN_ >= 256) ? 4 : (BN_ >= 128 ? 6 : 8));
+    // The fused error epilogue reads a tile of A after the MMAs, the comparing
+    // one is as long as they; two stages leave room for a second CTA on the SM,
+    // whose MMAs overlap that.
+    static constexpr int STAGES = (EPI != EPI_STORE) ? 2 : ((BN_ >= 256) ? 4 : (BN_ >= 128 ? 6 : 8));
     static constexpr int SMEM = STAGES * STAGE + 1024 /*align*/ + 256 /*barriers*/;
     static constexpr uint32_t TMEM_COLS = BN_ < 32 ? 32 : BN_;
 };
 
 template <bool A_MN, int BN_, int EPI, bool TF32>
-__global__ void __launch_bounds__(NTHREADS, EPI == EPI_ERR ? 2 : 1) tc_gemm_kernel(const __grid_constant__ Maps maps,
+__global__ void __launch_bounds__(NTHREADS, EPI != EPI_STORE ? 2 : 1) tc_gemm_kernel(const __grid_constant__ Maps maps,
                                                                                    Params p) {
     static_assert(!(TF32 && A_MN), "TF32 operands are K-major");
     using C = Cfg<A_MN, BN_, EPI>;
@@ -272,6 +275,30 @@ __global__ void __launch_bounds__(NTHREADS, EPI == EPI_ERR ? 2 : 1) tc_gemm_kern
         if (lane == 0) red[q] = local;
         asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
         if (warp == 2 && lane == 0) p.errp[blockIdx.x + (int64_t)blockIdx.y * gridDim.x] = red[0] + red[1] + red[2] + red[3];
+    } else if (warp >= 2 && EPI == EPI_COVER) {
+        // ---------------- comparing epilogue ----------------
+        const int q = warp & 3;
+        const int64_t row = m0 + 32 * q + lane;
+        const float2 need = row < p.M ? p.row_need[row] : make_float2(0.f, 0.f);
+        __shared__ float2 cn[BN_];
+        for (int c = threadIdx.x - 64; c < BN_; c += 128)
+            cn[c] = n0 + c < p.N ? p.col_need[n0 + c] : make_float2(0.f, 0.f);
+        asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
+        const bool got = __all_sync(0xffffffffu, mbar_wait(tmem_full, 0) ? 1 : 0) != 0;
+        if (!got) atomicExch(p.err_flag, 1);
+        tc_fence_after();
+        bool low = false;
+        if (got && iters > 0) {
+#pragma unroll 1
+            for (int c = 0; c < BN_; c += 16) {
+                float v[16];
+                tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c, v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j)   // nothing is needed beyond M and N; a NaN counts as low
+                    low |= !(v[j] >= fmaf(need.x, cn[c + j].x, need.y * cn[c + j].y));
+            }
+        }
+        if (low) *p.low = 1;
     } else if (warp >= 2) {
         // ---------------- store epilogue ----------------
         const int q = warp & 3;   // TMEM lane quarter this warp may access
@@ -531,6 +558,10 @@ cudaError_t tc_gemm_run(const TcGemmDesc &g, Scratch *ws, cudaStream_t s) {
     p.R = g.ref;
     p.ldr = g.ldref;
     p.errp = g.err_partials;
+    p.row_need = g.row_need;
+    p.col_need = g.col_need;
+    p.low = g.low;
+    if (g.epilogue == EPI_COVER && (g.tf32 || g.a_mn_major)) return cudaErrorInvalidValue;
     const int64_t tiles = ((g.M + BM - 1) / BM) * ((g.N + bn - 1) / bn);
     int splits = 1;
     if (g.epilogue == EPI_STORE && tiles < kNumSMs && p.kblocks >= 8) {
@@ -548,9 +579,10 @@ cudaError_t tc_gemm_run(const TcGemmDesc &g, Scratch *ws, cudaStream_t s) {
     p.kblocks_per_split = (p.kblocks + splits - 1) / splits;
     // the method's flops: one product (the split's extra pairs are the
     // implementation's overhead, not counted)
-    const double flops = 2.0 * g.M * g.N * g.K;
+    // (a comparison's are none of them)
+    const double flops = g.epilogue == EPI_COVER ? 0.0 : 2.0 * g.M * g.N * g.K;
     const double bytes = (g.tf32 ? 4.0 : 2.0) * g.npairs * ((double)g.M * g.K + (double)g.K * g.N) +
-                         (g.epilogue == EPI_ERR ? 4.0 * g.M * g.N : 4.0 * g.M * g.N);
+                         (g.epilogue == EPI_COVER ? 0.0 : 4.0 * g.M * g.N);
     ProfScope prof(PROF_TC_GEMM, flops, bytes, s);
     if (splits > 1) {
         p.D = part;
@@ -569,6 +601,8 @@ cudaError_t tc_gemm_run(const TcGemmDesc &g, Scratch *ws, cudaStream_t s) {
     if (g.tf32)
         e = g.epilogue == EPI_ERR ? launch_bn<false, EPI_ERR, true>(bn, maps, p, 1, s)
                                   : launch_bn<false, EPI_STORE, true>(bn, maps, p, splits, s);
+    else if (g.epilogue == EPI_COVER)
+        e = launch_bn<false, EPI_COVER, false>(bn, maps, p, 1, s);
     else if (g.epilogue == EPI_ERR)
         e = g.a_mn_major ? launch_bn<true, EPI_ERR, false>(bn, maps, p, 1, s)
                          : launch_bn<false, EPI_ERR, false>(bn, maps, p, 1, s);

@@ -23,6 +23,8 @@ struct TcOperand {
 // K, outer = M) unless a_mn_major, then inner = M and outer = K.
 // EPI_ERR: instead of storing D, each CTA writes sum((ref - D)^2) over its
 // tile to err_partials[cta] (tc_gemm_err_ctas() entries).
+// EPI_COVER: instead of storing D, sets *low where an entry is not at least
+// row_need[i].x col_need[j].x + row_need[i].y col_need[j].y (BF16, K-major).
 struct TcGemmDesc {
     int64_t M = 0, N = 0, K = 0;
     bool a_mn_major = false;
@@ -35,6 +37,8 @@ struct TcGemmDesc {
     const float *ref = nullptr;
     int64_t ldref = 0;
     double *err_partials = nullptr;
+    const float2 *row_need = nullptr, *col_need = nullptr;
+    int *low = nullptr;
     int *err_flag = nullptr;      // set to 1 by a CTA whose bounded wait ran out
     int bn = 0;                   // N tile (32, 64, 128, 256); 0 = by N
     float alpha = 1.f, beta = 0.f;
