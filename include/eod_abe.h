@@ -274,6 +274,11 @@ EOD_API eod_status eod_abe_debug_profile_read(int32_t kind, int64_t *launches, d
                                               double *total_flops, double *total_bytes);
 EOD_API int64_t eod_abe_debug_launch_count(void);
 
+/* Test hook (no counterpart in the paper): the side streams the library has
+ * created (for work that overlaps a factorisation's own stream) and not
+ * destroyed; at most as many as calls ran at the same time, or 64 idle ones. */
+EOD_API int64_t eod_abe_debug_side_streams(void);
+
 /* Test hook (no counterpart in the paper): one tcgen05 tensor-core
  * contraction of the mixed path on FP32 device inputs, split into BF16
  * hi/lo parts inside the call.  All matrices column-major.

@@ -35,7 +35,7 @@ EXPORTED = [
     "eod_abe_debug_profile_read", "eod_abe_debug_launch_count", "eod_abe_fro_norm_noalloc",
     "eod_abe_debug_tc_gemm", "eod_abe_debug_f64_gemm", "eod_abe_debug_chol", "eod_abe_debug_bounded_wait",
     "eod_abe_debug_recip", "eod_abe_tuning_load", "eod_abe_tuning_lookup", "eod_abe_debug_f32_gemm",
-    "eod_abe_debug_batch_phases",
+    "eod_abe_debug_batch_phases", "eod_abe_debug_side_streams",
 ]
 
 
@@ -113,6 +113,8 @@ def _load() -> ctypes.CDLL:
     lib.eod_abe_debug_profile_read.restype = I32
     lib.eod_abe_debug_launch_count.argtypes = []
     lib.eod_abe_debug_launch_count.restype = I64
+    lib.eod_abe_debug_side_streams.argtypes = []
+    lib.eod_abe_debug_side_streams.restype = I64
     lib.eod_abe_fro_norm_noalloc.argtypes = [P, I64, I64, I64, I32, P, P, P]
     lib.eod_abe_fro_norm_noalloc.restype = I32
     lib.eod_abe_debug_tc_gemm.argtypes = [I32, I64, I64, I64, P, I64, P, I64, P, I64, P, P]
@@ -157,6 +159,7 @@ eod_abe_version = _lib.eod_abe_version
 eod_abe_debug_profile = _lib.eod_abe_debug_profile
 eod_abe_debug_profile_read = _lib.eod_abe_debug_profile_read
 eod_abe_debug_launch_count = _lib.eod_abe_debug_launch_count
+eod_abe_debug_side_streams = _lib.eod_abe_debug_side_streams
 eod_abe_fro_norm_noalloc = _lib.eod_abe_fro_norm_noalloc
 eod_abe_debug_tc_gemm = _lib.eod_abe_debug_tc_gemm
 eod_abe_debug_bounded_wait = _lib.eod_abe_debug_bounded_wait

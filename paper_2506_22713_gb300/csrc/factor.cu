@@ -473,22 +473,75 @@ static bool core_one_leaf(int64_t r) {
     return r <= 128 && !(tuned_value("core_leaf", r, 0, 0, &v) && v < r);
 }
 
-// A non-blocking stream of the calling thread on the current device, for
-// work that overlaps the main stream of a factorisation (created once per
-// thread and device, kept for the life of the process).
-static cudaStream_t side_stream() {
-    thread_local cudaStream_t streams[64] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        cudaGetLastError();
-        return nullptr;
+// Non-blocking streams for work that overlaps the main stream of a
+// factorisation.  A call leases one of its device; given back, it serves the
+// next call of any thread (a stream per thread is lost with the thread, and the
+// batched form makes new ones in every call).  At most kMost idle ones stay.
+// Work still queued on a stream given back only delays its next holder, whose
+// streams are ordered by events of its own.
+class SideStreams {
+public:
+    cudaStream_t take(int dev) {
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            for (size_t i = free_.size(); i-- > 0;)
+                if (free_[i].first == dev) {
+                    cudaStream_t st = free_[i].second;
+                    free_.erase(free_.begin() + i);
+                    return st;
+                }
+        }
+        cudaStream_t st = nullptr;
+        if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        alive_.fetch_add(1);
+        return st;
     }
-    if (!streams[dev] && cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        streams[dev] = nullptr;
+    void give(int dev, cudaStream_t st) {
+        {
+            std::lock_guard<std::mutex> lk(mu_);
+            if (free_.size() < kMost) {
+                free_.emplace_back(dev, st);
+                return;
+            }
+        }
+        cudaStreamDestroy(st);
+        alive_.fetch_sub(1);
     }
-    return streams[dev];
+    int64_t alive() const { return alive_.load(); }
+
+private:
+    static constexpr size_t kMost = 64;   // as many as the batched form has worker streams at most
+    std::mutex mu_;
+    std::vector<std::pair<int, cudaStream_t>> free_;
+    std::atomic<int64_t> alive_{0};
+};
+static SideStreams &side_streams() {
+    static SideStreams *p = new SideStreams;   // lives as long as the process: calls may come from exiting threads
+    return *p;
 }
+
+// One call's side stream, created when first asked for (null: none to be had).
+struct SideStream {
+    int dev = -1;
+    cudaStream_t st = nullptr;
+    SideStream() = default;
+    SideStream(const SideStream &) = delete;
+    SideStream &operator=(const SideStream &) = delete;
+    ~SideStream() {
+        if (st) side_streams().give(dev, st);
+    }
+    cudaStream_t get() {
+        if (st) return st;
+        if (cudaGetDevice(&dev) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return st = side_streams().take(dev);
+    }
+};
 
 // Makes `main` wait for everything queued on `side` so far, when it goes out
 // of scope (on every return path): the buffers both streams use are freed on
@@ -561,6 +614,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
 
     HostMirror hm(s);
     EOD_TRY(hm.init());
+    SideStream side;   // outlives the joins below
 
     // ---- workspace ----
     Scratch ws;
@@ -740,7 +794,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     // (only where the sketch has work enough to hide: for small problems the
     // extra buffers and events cost more than the leaf they overlap;
     // EOD_LOOKAHEAD=0 / 1 turns it off / on regardless of size)
-    cudaStream_t s2 = cap > k ? side_stream() : nullptr;
+    cudaStream_t s2 = cap > k ? side.get() : nullptr;
     bool lookahead = s2 != nullptr && s2 != s && (double)m * (double)n >= 4.0e6;
     if (const char *env = std::getenv("EOD_LOOKAHEAD")) lookahead = s2 != nullptr && s2 != s && env[0] == '1';
     T *Y2 = nullptr, *S2 = nullptr, *Om2 = nullptr;
@@ -1013,7 +1067,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     JoinOnExit join;
     if (o.compute_err) {
         Phase ph("eod.reconstruction_error");
-        cudaStream_t se = side_stream();
+        cudaStream_t se = side.get();
         if (!se) se = s;
         join.main = s;
         if (mixed) {
@@ -1541,6 +1595,8 @@ double eod_abe_model_flops(int64_t m, int64_t n, int64_t r, int64_t k, int32_t w
     if (with_err) f += 2.0 * M * N * Rr;
     return f;
 }
+
+int64_t eod_abe_debug_side_streams(void) { return side_streams().alive(); }
 
 void eod_abe_debug_fail_alloc_after(int32_t n) { g_fail_alloc_after = n > 0 ? n : 0; }
 
