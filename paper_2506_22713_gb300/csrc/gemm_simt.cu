@@ -561,13 +561,12 @@ int64_t gemm_err_ctas(int64_t M, int64_t N) { return ((M + BM - 1) / BM) * ((N +
 // block.  Whole factorisations in blocks of 32 without / with them: 716 x 716,
 // rank 13 489 / 514 us, rank 102 1441 / 1376; 620 x 900, rank 20 568 / 575;
 // 800 x 800, rank 30 660 / 607; 1000 x 1000, rank 30 728 / 624.
-static int fp64_mode() {   // 0 SIMT always, 1 by size, 2 emulation always
-    static const int mode = [] {
-        const char *v = std::getenv("EOD_FP64_GEMM");
-        if (v && std::strcmp(v, "simt") == 0) return 0;
-        if (v && std::strcmp(v, "emulated") == 0) return 2;
-        return 1;
-    }();
+static int emulation_mode(const char *name) {   // 0 SIMT always, 1 by size, 2 emulation always
+    const char *v = std::getenv(name);
+    return v && std::strcmp(v, "simt") == 0 ? 0 : v && std::strcmp(v, "emulated") == 0 ? 2 : 1;
+}
+static int fp64_mode() {
+    static const int mode = emulation_mode("EOD_FP64_GEMM");
     return mode;
 }
 static bool fp64_emulate(int64_t M, int64_t N, int64_t K, double least, int64_t side) {
@@ -583,21 +582,21 @@ bool fp64_emulate_product(int64_t M, int64_t N, int64_t K, double frac) {
     return fp64_use_emulated(M, N, K) || fp64_emulate(M, N, K, 2.1e7 / frac, 64);
 }
 
-// Large FP32 products go to the emulation with four digits (oz_gemm.cu), whose
-// result is the exact product's rounding (relative error 2.5e-8; FFMA 1e-7 to
-// 1.3e-6), where neither side is narrow: its tiles are 128 x 64 and both
-// operands are sliced on every call.  FFMA against digits with their slicing:
+// Large FP32 products go to the emulation with four digits (oz_gemm.cu) where
+// neither side is narrow: its tiles are 128 x 64 and both operands are sliced
+// on every call.  Its error is about 2^-31 of row scale x column scale per term,
+// and the result is rounded once: on dense operands 2.5e-8 relative (FFMA 1e-7
+// to 1.3e-6), on entries whose own terms are below 2^-7 of the scales more than
+// FFMA's.  The products of a factorisation have results accurate in norm only;
+// A_hat is checked entry by entry.  FFMA against digits with their slicing:
 // 8192 x 8192 x 473 1515 / 875 us, 3001 x 2503 x 313 306 / 140, 2049 x 326 x
 // 1537 299 / 96, 8192 x 455 x 8192 1936 / 1144, 8192 x 455 x 455 115 / 104; and
 // below the line 8192 x 256 x 256 35 / 61, 2503 x 313 x 313 44 / 61, 8192 x 96 x
-// 384 49 / 73, 2048 x 2048 x 64 21 / 76.  EOD_FP32_GEMM=emulated sends every
-// product there.
+// 384 49 / 73, 2048 x 2048 x 64 21 / 76.  EOD_FP32_GEMM=simt keeps all on FFMA,
+// =emulated sends every product to the digits.
 bool fp32_use_emulated(int64_t M, int64_t N, int64_t K) {
-    static const bool all = [] {
-        const char *v = std::getenv("EOD_FP32_GEMM");
-        return v && std::strcmp(v, "emulated") == 0;
-    }();
-    if (all) return M >= 1 && N >= 1 && K >= 1;
+    static const int mode = emulation_mode("EOD_FP32_GEMM");
+    if (mode != 1) return mode == 2 && M >= 1 && N >= 1 && K >= 1;
     return M >= 256 && N >= 256 && K > 256 && (double)M * (double)N * (double)K >= 7.6e8;   // 2^29.5
 }
 
