@@ -63,7 +63,8 @@ def tuned_k(form, m, n, default=32):
 
 # FP64 peak from unit counts and clock: 152 SMs x 2 DFMA/clk/SM x 2 flop x 2070 MHz
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.070
-FP64_SM_PEAK_GFLOPS = FP64_PEAK_GFLOPS / 152
+# ... of the eight SMs that a leaf's cluster takes (up to 16 columns it takes one)
+FP64_SM_PEAK_GFLOPS = FP64_PEAK_GFLOPS / 152 * 8
 # FP32 (FFMA) peak: 152 SMs x 128 lanes x 2 flop x 2070 MHz
 FP32_PEAK_GFLOPS = 152 * 128 * 2 * 2.070
 L2_BYTES = 129 * 1024 * 1024
@@ -265,8 +266,8 @@ def roofline_of(kind, rec, peaks):
     elif kind == "chol":
         ach = fl / (ms / 1e3) / 1e9
         out.update(bound="alu", achieved=ach, peak=FP64_SM_PEAK_GFLOPS, unit="GFLOP/s",
-                   peak_source="FP64 of one SM from unit counts: 2 DFMA/clk x 2 flop x 2070 MHz (the kernel is one "
-                               "CTA)")
+                   peak_source="FP64 of the leaf's eight SMs (a cluster; one up to 16 columns) from unit counts: "
+                               "2 DFMA/clk x 2 flop x 2070 MHz each")
     elif kind == "gemm_simt":
         ach = fl / (ms / 1e3) / 1e9
         out.update(bound="alu", achieved=ach, peak=FP64_PEAK_GFLOPS, unit="GFLOP/s",

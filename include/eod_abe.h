@@ -59,17 +59,22 @@ typedef enum { EOD_F64 = 0, EOD_F32 = 1 } eod_dtype;
 
 typedef enum {
     EOD_PLAIN = 0,         /* every contraction at the precision of A's storage
-                              type.  EOD_F64: products of at least 2^25
-                              multiply-adds run as an exact FP64 emulation on
-                              the tcgen05 tensor cores (each operand split into
-                              seven BF16 digit slices, integer-exact partial
-                              products and sums, one rounding; normwise error
-                              about K 2^-54 |A(i,:)| |B(:,j)|), smaller ones as
-                              FP64 DFMA; EOD_F32: FP32 FFMA, the products with
-                              no narrow side and 2^29.5 multiply-adds or more
-                              as the same emulation with four digits, rounded
-                              once to FP32.  Gram/Cholesky/rank test/core in
-                              FP64 */
+                              type.  EOD_F64: larger products (from 1.2e7 to
+                              2^25 multiply-adds on, by what has to be split
+                              for them; all from 2^25 on) run as an FP64
+                              emulation on the tcgen05 tensor cores (each
+                              operand split into seven BF16 digit slices,
+                              integer-exact partial products and sums, one
+                              rounding; error per term about 2^-55 of the
+                              largest entry of A's row times that of B's
+                              column), smaller ones as FP64 DFMA; EOD_F32: FP32
+                              FFMA, the products with no narrow side and 2^29.5
+                              multiply-adds or more as the same emulation with
+                              four digits (2^-31 of those scales per term),
+                              rounded once to FP32.  Gram/Cholesky/rank
+                              test/core in FP64.  The environment variables
+                              EOD_FP64_GEMM and EOD_FP32_GEMM (read once) set to
+                              "simt" keep all products on the FMAs */
     EOD_MIXED_BF16 = 1,    /* sketch, projection and reconstruction on tcgen05
                               tensor cores with FP32 accumulation: A split into
                               three BF16 terms for the sketch (exact for FP32
@@ -173,7 +178,9 @@ EOD_API eod_status eod_abe_factor_host(const void *A_host, int64_t m, int64_t n,
 
 /* Rebuilds A_hat = U D V^T, the product of the three factors (paper Sec. 1),
  * into device buffer A_hat (m x n, ld ld_hat >= m), written in opts->a_dtype
- * (NULL opts: the factors' f_dtype).  Rank 0 writes zeros.  Errors:
+ * (NULL opts: the factors' f_dtype).  Rank 0 writes zeros.  Every entry is as
+ * accurate as FMA products make it, |error| <= 2 (r + 2) u (|U| |D| |V|^T): large
+ * ones run on the tensor cores only where that is sure to hold.  Errors:
  * EOD_EINVAL for NULL f or A_hat or ld_hat < m; EOD_EUNSUPPORTED when the
  * requested type differs from f_dtype. */
 EOD_API eod_status eod_abe_reconstruct(const eod_factors *f, void *A_hat, int64_t ld_hat,
@@ -245,10 +252,10 @@ EOD_API void eod_abe_debug_fail_alloc_after(int32_t n);
 /* Measurement hooks (no counterpart in the paper; they support the
  * benchmark's roofline figures).
  * eod_abe_debug_profile(1) clears and starts CUDA-event timing of every
- * kernel launch, grouped by kind: 0 SIMT GEMM, 1 one-CTA Cholesky / rank
+ * kernel launch, grouped by kind: 0 SIMT GEMM, 1 leaf Cholesky / rank
  * test, 2 Omega generation, 3 streaming (norms, copies, splitting),
- * 4 tcgen05 tensor-core GEMM (mixed path), 5 FP64 GEMM emulated on tcgen05
- * (plain FP64 path), 6 slicing of FP64 operands into the BF16 digits of that
+ * 4 tcgen05 tensor-core GEMM (mixed path), 5 FP64 (and large FP32) GEMM
+ * emulated on tcgen05, 6 slicing of operands into the BF16 digits of that
  * emulation, 7 SIMT GEMM and Gram in FP32 arithmetic (FP32-data paths; kind 0
  * is then the FP64 ones), 8 the persistent batched launch (one record per
  * launch); eod_abe_debug_profile(0) stops it and clears.
@@ -353,7 +360,8 @@ EOD_API eod_status eod_abe_debug_chol(const double *G, int64_t ldg, int32_t w, i
                                       int64_t ldr, int32_t *info, void *stream);
 
 /* Test hook (no counterpart in the paper): the reciprocal the leaf
- * factorisation (eod_abe_debug_chol, Alg. 1 steps 5-11) takes of each pivot,
+ * factorisation on one CTA (eod_abe_debug_chol up to 16 columns, the batched
+ * form; Alg. 1 steps 5-11) takes of each pivot,
  * applied to n device doubles d (out[i] = 1/d[i], FP64, device memory):
  * seeded by an FP32 reciprocal of the mantissa and refined by one
  * third-order step, within 2 ulp of 1/d for normal d whose reciprocal is
@@ -366,7 +374,7 @@ EOD_API eod_status eod_abe_debug_recip(const double *d, double *out, int64_t n, 
  * op(B) + beta C on device matrices, column-major, op(X) = X^T when the
  * matching flag is nonzero; mode & 3 == 0 runs the SIMT DFMA kernel, 1 the
  * FP64 emulation on tcgen05 tensor cores that the plain FP64 path uses for
- * large products (exact BF16 slices, FP64 accumulation).  Bits of mode above
+ * large products (BF16 digit slices, exact sums, one rounding).  Bits of mode above
  * those select the structured forms the factorisation uses: 16 = only the
  * upper triangle of C is wanted (the emulation stores row <= col only, the
  * SIMT kernel whole tiles that touch it), 32 = op(A) upper triangular,

@@ -87,7 +87,7 @@ cudaError_t chol_small(const double *G, int64_t ldg, int w, int decide, double e
                        cudaStream_t s, double ni_tau2, bool classic, const CholOut &out) {
     if (w < 1 || w > 128) return cudaErrorInvalidValue;
     if (decide || shift != 0.0) ni_tau2 = 0.0;
-    ProfScope prof(PROF_CHOL, (double)w * w * w * (Rinv ? 2.0 : 1.0) / 3.0, sizeof(double) * 3.0 * w * w, s);
+    ProfScope prof(PROF_CHOL, (double)w * w * w * (Rinv || out.RinvF ? 2.0 : 1.0) / 3.0, sizeof(double) * 3.0 * w * w, s);
     count_launch();
     const LeafArgs args{G, ldg, w, decide, eps2, delta_coef, rho, shift, R, ldr, Rinv, ldinv, out.RinvF, out.ldf, info,
                         ni_tau2, out.tR1, out.tdiag};

@@ -183,7 +183,7 @@ cudaError_t gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha
 int64_t gemm_err_ctas(int64_t M, int64_t N);
 
 // FP64 GEMM emulated on tcgen05 tensor cores (oz_gemm.cu); same contract as
-// gemm<double,...> except that the triangular / upper-only hints are ignored
+// gemm<double,...>; upper_only stores row <= col alone
 cudaError_t oz_gemm(bool ta, bool tb, int64_t M, int64_t N, int64_t K, double alpha, const double *A, int64_t lda,
                     const double *B, int64_t ldb, double beta, double *C, int64_t ldc, const GemmExtra &x,
                     int *err_flag, cudaStream_t s);
@@ -267,7 +267,7 @@ cudaError_t gram_tiled_f32(const float *W, int64_t rows, int64_t p, int64_t ldw,
                            Scratch *ws, cudaStream_t s);
 
 // --------------------------------------------------------------------------
-// Small dense factorisations (one CTA)
+// Small dense factorisations (one CTA up to 16 columns, else a cluster of eight)
 // --------------------------------------------------------------------------
 enum CholCode { CHOL_ALL = 0, CHOL_BELOW = 1, CHOL_UNCERTAIN = 2, CHOL_FAIL = 3 };
 

@@ -147,7 +147,7 @@ template <> struct Traits<float> { static constexpr int dtype = EOD_F32; static 
 // Blocked CholQR pass on W (rows x p, FP64 Gram, FP64 R):  G = W^T W,
 // R = chol(G + shift I), W <- W R^{-1}.
 // The Cholesky runs right-looking over panels of kPB columns: each diagonal
-// panel is factored left-looking over 64-column leaves (one CTA each, the
+// panel is factored left-looking over 64-column leaves (a cluster each, the
 // leaf inverses kept), its triangular inverse formed, then the panel row of R
 // and the trailing Gram update are two large products.  The solve
 // W <- W R^{-1} runs over the same panels (diagonal inverse, then the
@@ -786,7 +786,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
     };
 
     // Lookahead across blocks: while block j's Gram and rank-test leaf run
-    // (one CTA), the next block is sketched and given its first projection
+    // (eight CTAs at most), the next block is sketched and given its first projection
     // pass against the basis that existed before block j, on a side stream
     // with its own buffers; block j+1 then only projects out block j's own
     // columns before its second pass (the same BCGS2 result in exact
@@ -1085,8 +1085,7 @@ static eod_status factor_impl(const T *A, int64_t m, int64_t n, int64_t lda, dou
                 EOD_TRY(ar.get(&cts, (size_t)kOzSlices * n * r8));
                 EOD_TRY(ar.get(&ects, (size_t)n));
             }
-            // the SIMT path takes split-K partials from the shared workspace:
-            // only the emulated product (no workspace use) leaves `s`
+            // only the product with Q's kept slices leaves `s`
             if (!emulated) se = s;
             join.side = se;
             EOD_CU(stream_after(se, s));

@@ -1,13 +1,12 @@
 // SIMT GEMM of the plain (FP64 / FP32) path: the dense contractions of
-// Alg. 1 and Alg. 2 that do not go to the tensor cores.  With FP32 data that
-// is all of them but the core's large Gram matrices (widened to FP64 and
-// emulated in oz_gemm.cu): the sketch A*Omega of Alg. 1 step 4, the two block
-// Gram-Schmidt projections Q^T Y and Y - Q S of step 4, the CholQR Grams of
-// step 5, the projection C^T = A^T Q of Alg. 2 step 8, the triangular solves
-// and products of steps 9-11 and the reconstruction Q C with its fused
-// Frobenius error of Sec. 4.1.  With FP64 data only the products below 2^25
-// multiply-adds (and the CGS2 residual's matrix-vector products) run here:
-// the larger ones are the FP64 emulation on tcgen05 in oz_gemm.cu.
+// Alg. 1 and Alg. 2 that do not go to the tensor cores (the sketch A*Omega and
+// the two block Gram-Schmidt projections Q^T Y and Y - Q S of Alg. 1 step 4, the
+// projection C^T = A^T Q of Alg. 2 step 8, the triangular solves and products of
+// steps 9-11, the reconstruction Q C with its fused Frobenius error of Sec. 4.1,
+// the CGS2 residual's matrix-vector products), and the rules that send the
+// larger ones to the emulation in oz_gemm.cu: FP64 products by size and by what
+// has to be sliced, FP32 ones from 2^29.5 multiply-adds without a narrow side,
+// FP32 data's wide Grams widened to FP64.
 //
 // Tile TS x TS x 16 (TS = 64, 32 or 16: the smaller tiles spread products too
 // small to fill the 152 SMs with 64-tiles), 256 threads, (TS/16)^2 outputs
@@ -557,6 +556,9 @@ int64_t gemm_err_ctas(int64_t M, int64_t N) { return ((M + BM - 1) / BM) * ((N +
 //   512 x 256 x 64      22 /  29 / 24     1000 x 32 x 1000    72 / 50 / 26
 //   256 x 256 x 256     39 /  44 / 24     512 x 32 x 384      26 / 40 / 22
 //   1000 x 104 x 1000  200 /  53 / 28     2048 x 128 x 128    65 / 42 / 27
+// "Without that of the first" holds for S = Q^T Y, whose slices have a column's
+// own exponent; products with Q's rows (one exponent for all) take the line of
+// 2^25 (factor.cu).
 // Keeping slices of A and Q costs two passes over A and two small launches per
 // block.  Whole factorisations in blocks of 32 without / with them: 716 x 716,
 // rank 13 489 / 514 us, rank 102 1441 / 1376; 620 x 900, rank 20 568 / 575;

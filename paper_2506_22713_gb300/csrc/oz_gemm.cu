@@ -44,13 +44,15 @@
 // (four per TMEM lane quarter, 16 columns each).  All waits are bounded
 // (EOD_ETIMEOUT on expiry).
 //
-// Measured (the kernel alone): 2048^3 373 us = 46 TFLOP/s of FP64, 4000 x 1600
-// x 1600 459 us, 4000 x 1600 x 4000 999 us.  With one MMA of 64 columns per
-// slice pair (72 cycles each instead of 32: shared-memory reads, 6 KB per MMA),
-// eight drain warps and one hand-over per chunk: 634, 776 and 1750 us; wide MMAs
-// alone 452, 563 and 1209; with sixteen drain warps 429, 530 and 1173.  What
-// bounds it now: shared-memory reads (4.4 thousand cycles of a K block's about
-// 5, the MMAs alone 3.6), the first and last chunk's drain, and the last wave
+// Measured (the kernel alone): 2048^3 391 us = 44 TFLOP/s of FP64, 4000 x 1600
+// x 1600 479 us, 4000 x 1600 x 4000 1053 us; with both halves handed over every
+// 256 terms, where the upper groups' sums could pass 2^24, 373, 459 and 999.  In
+// that form, with one MMA of 64 columns per slice pair (72 cycles each instead
+// of 32: shared-memory reads, 6 KB per MMA), eight drain warps and one hand-over
+// per chunk: 634, 776 and 1750 us; wide MMAs alone 452, 563 and 1209; with
+// sixteen drain warps 429, 530 and 1173.  What bounds it: shared-memory reads
+// (4.4 thousand cycles of a K block's about 5, the MMAs alone 3.6), the drains
+// that the next products wait for, the first and last chunk's, and the last wave
 // of tiles.  Slicing a 2048^2 operand and its transpose: 57 us.
 #include "common.cuh"
 #include "instrument.cuh"
