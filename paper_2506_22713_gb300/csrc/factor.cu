@@ -58,6 +58,7 @@ static eod_status cuda_status(cudaError_t e) {
 // factorisation.  A block belongs to one call at a time; at most kMost stay.
 class PinnedBlocks {
 public:
+    PinnedBlocks() { free_.reserve(kMost); }   // nothing is allocated when one is given back
     void *take() {
         {
             std::lock_guard<std::mutex> lk(mu_);
@@ -481,6 +482,7 @@ static bool core_one_leaf(int64_t r) {
 // streams are ordered by events of its own.
 class SideStreams {
 public:
+    SideStreams() { free_.reserve(kMost); }   // nothing is allocated when one is given back
     cudaStream_t take(int dev) {
         {
             std::lock_guard<std::mutex> lk(mu_);

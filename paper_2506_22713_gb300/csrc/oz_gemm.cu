@@ -886,7 +886,7 @@ template <int NS>
 cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N, int64_t K, double alpha, double beta,
                     double *C, int64_t ldc, const GemmExtra &x, int *err_flag, cudaStream_t s, float *Cf) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    if ((NS == kOzSlicesF32) != (Cf != nullptr) || (Cf && x.epilogue != EPI_STORE)) return cudaErrorInvalidValue;
+    if ((NS == kOzSlicesF32) != (Cf != nullptr) || (NS != kOzSlices && x.epilogue != EPI_STORE)) return cudaErrorInvalidValue;
     cudaError_t e = cudaSuccess;
     Maps maps;
     std::memset(&maps, 0, sizeof(maps));
@@ -933,7 +933,7 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
     double *part = nullptr;
     constexpr int SMEM = Cfg<NS>::SMEM;
     e = set_smem_once(oz_gemm_kernel<NS, EPI_STORE>, SMEM);
-    if constexpr (NS != kOzSlicesF32)
+    if constexpr (NS == kOzSlices)
         if (e == cudaSuccess) e = set_smem_once(oz_gemm_kernel<NS, EPI_ERR>, SMEM);
     if (e == cudaSuccess && splits > 1) {
         e = room((void **)&part, sizeof(double) * (size_t)splits * M * N, s);
@@ -962,7 +962,7 @@ cudaError_t run_ops(const OzOperand &A, const OzOperand &B, int64_t M, int64_t N
             grid = dim3(kNumSMs);
         }
         count_launch();
-        if constexpr (NS == kOzSlicesF32) {
+        if constexpr (NS != kOzSlices) {
             oz_gemm_kernel<NS, EPI_STORE><<<grid, NTHREADS, SMEM, s>>>(maps, p);
         } else {
             if (x.epilogue == EPI_ERR) oz_gemm_kernel<NS, EPI_ERR><<<grid, NTHREADS, SMEM, s>>>(maps, p);
